@@ -91,6 +91,12 @@ int check_device_ptr(hts_ctx *c, const void *p)
     return HTS_OK;
 }
 
+__global__ void empty_nodes_kernel(int64_t slots, NodeF *nodes)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < slots) nodes[k] = NodeF{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, (int)(k + 1)};
+}
+
 int ensure_points(hts_ctx *c, int64_t n)
 {
     if (n == c->cap_n && (c->pts32 || c->pts64)) return HTS_OK;
@@ -117,9 +123,12 @@ int ensure_points(hts_ctx *c, int64_t n)
         AL(c->nodes64, 2 * N);
     }
     // a node slot never written by a tree build reads as an empty bucket
-    // (count 0), which the walk steps over
-    if (c->nodes32 && cudaMemset(c->nodes32, 0, sizeof(NodeF) * (2 * N + kWalkOverrun)) != cudaSuccess)
-        return HTS_ECUDA;
+    // (count 0), which the walk steps over (its skip is its index + 1)
+    if (c->nodes32) {
+        const int64_t slots = (int64_t)(2 * N + kWalkOverrun);
+        empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256>>>(slots, c->nodes32);
+        if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return HTS_ECUDA;
+    }
     if (c->nodes64 && cudaMemset(c->nodes64, 0, sizeof(NodeD) * 2 * N) != cudaSuccess) return HTS_ECUDA;
     AL(c->keys, N);
     AL(c->keys_alt, N);
@@ -164,6 +173,12 @@ int ensure_points(hts_ctx *c, int64_t n)
         }
         c->split_part = part;
         c->split_frontier = fr;
+    }
+    if (c->cfg.precision == HTS_FP32_MIXED) {
+        const size_t pages = (size_t)list_pages((int64_t)N);
+        AL(c->list_entries, pages * (list_page_bytes() / sizeof(uint2)));
+        AL(c->list_head, pages);
+        AL(c->list_flags, (size_t)list_flags((int64_t)N));
     }
 #undef AL
     c->n_nodes = c->pre + n;
@@ -511,6 +526,7 @@ void hts_destroy(hts_ctx *c)
     dfree(&c->bn_lo); dfree(&c->bn_hi); dfree(&c->bn_pref); dfree(&c->bn_flag); dfree(&c->bn_quad);
     dfree(&c->bn_sum); dfree(&c->cnt); dfree(&c->pre); dfree(&c->nodes32); dfree(&c->apts32); dfree(&c->walk_cost); dfree(&c->walk_order); dfree(&c->nodes64);
     dfree(&c->sort_scratch); dfree(&c->scan_tmp); dfree(&c->exact_part);
+    dfree(&c->list_entries); dfree(&c->list_head); dfree(&c->list_flags);
     if (c->split_part) cudaFree(c->split_part);
     if (c->split_frontier) cudaFree(c->split_frontier); dfree(&c->red_tmp); dfree(&c->minmax);
     dfree(&c->dscal); dfree(&c->status); dfree(&c->counters); dfree(&c->xsq);

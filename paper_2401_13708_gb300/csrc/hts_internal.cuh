@@ -63,19 +63,22 @@ struct __align__(16) PointD {
 //                midpoint, thr = cosh(r_cell / theta) - 1 (accept iff the
 //                pair's delta = cosh(d) - 1 exceeds it), skip = pre-order
 //                index after the subtree.
-//   count == 1 : single-point leaf; the point itself, thr holds the point's
-//                sorted position (int bits), skip = index + 1.
-//   count <  0 : depth-29 bucket of -count points; thr holds the sorted
-//                position of its first point (int bits).
+//   count == 1 : single-point leaf; the point itself, thr = -1 (every delta
+//                exceeds it), skip = index + 1.
+//   count <  0 : depth-29 bucket of -count points, thr = -1; il holds the
+//                sorted position of its first point (int bits).
+// Every slot's skip exceeds its index, written by a tree build or not.
 struct __align__(16) NodeF {
     float xh, yh, xl, yl;
     float il, thr;
     float count;
     int skip;
 };
-// Empty float32 node slots the tree build writes after its last node (the
-// walk visits up to three past its last node: four visits per loop test).
-constexpr int kWalkOverrun = 4;
+// Visits of the float32 walk per test of its cursor (walk_f32_chunk), and the
+// empty node slots the tree build writes after its last node: the walk visits
+// up to kWalkTrip - 1 past its last node and loads one further.
+constexpr int kWalkTrip = 8;
+constexpr int kWalkOverrun = kWalkTrip + 1;
 
 // Tree node, float64 mode (same meaning; pos = sorted position for leaves
 // and buckets).
@@ -187,7 +190,10 @@ struct hts_ctx {
     int attract_background = 0;      // set while the attraction is launched beside the walk
     unsigned *walk_cost = nullptr;   // per walk block: cycles of the last walk (launch-order input)
     int *walk_order = nullptr;       // [0] grid size, then the launch order of the walk's blocks
-    void *split_frontier = nullptr;  // frontier table + entry count
+    void *split_frontier = nullptr;  // cuts of the tree (CutTables)
+    uint2 *list_entries = nullptr;   // interaction lists of the float32 walk: pages of 32 entries,
+    int2 *list_head = nullptr;       //   entries and next page of each page,
+    int *list_flags = nullptr;       //   pages taken per pool, then a flag per chunk
     void *split_part = nullptr;      // partial sums of the split walk
 
     // CO-SNE term (Sec. 4.3): lambda1 KL + lambda2 (1/n) sum (|x|^2 - |y|^2)^2
@@ -231,6 +237,10 @@ int exact_split(int64_t n);
 int walk_split_capacity(int64_t n);
 int walk_split_depth(int64_t n, int want, bool fp64);
 size_t walk_split_frontier_bytes();
+// interaction lists: pages for n points, bytes of a page, counters and flags
+int64_t list_pages(int64_t n);
+size_t list_page_bytes();
+int64_t list_flags(int64_t n);
 // attract.cu
 void launch_attract(hts_ctx *c);
 void launch_kl_terms(hts_ctx *c);
@@ -321,6 +331,52 @@ __device__ __forceinline__ PairF pair_terms_f32(float delta)
         p.rep = p.w * p.att;
     }
     return p;
+}
+
+// pair_terms_f32 of a delta known to be below its series limit (0.02): the same
+// operations on the series side, without the logarithm and the selection.
+template <int GF>
+__device__ __forceinline__ PairF pair_terms_small_f32(float delta)
+{
+    delta = fmaxf(delta, 1e-30f);
+    const float x = delta * (delta + 2.0f);
+    const float rs = rsqrtf(x);
+    const float t = x * rs;
+    float f = -2.0f / 35.0f;
+    f = fmaf(f, delta, 2.0f / 15.0f);
+    f = fmaf(f, delta, -1.0f / 3.0f);
+    f = fmaf(f, delta, 1.0f);
+    const float d = t * f;
+    PairF p;
+    p.w = __fdividef(1.0f, fmaf(d, d, 1.0f));
+    p.att = p.w * (GF == 0 ? f : rs);
+    p.rep = p.w * p.att;
+    return p;
+}
+
+// The pair terms w and rep of two deltas in paired float32 arithmetic, each
+// component with the operations and roundings of pair_terms_f32.
+template <int GF>
+__device__ __forceinline__ void pair_terms2_f32(float2 delta, float2 &w, float2 &rep)
+{
+    delta.x = fminf(fmaxf(delta.x, 1e-30f), 1e18f);
+    delta.y = fminf(fmaxf(delta.y, 1e-30f), 1e18f);
+    const float2 x = __fmul2_rn(delta, __fadd2_rn(delta, make_float2(2.0f, 2.0f)));
+    const float2 rs = make_float2(rsqrtf(x.x), rsqrtf(x.y));
+    const float2 t = __fmul2_rn(x, rs);
+    float2 fs = make_float2(-2.0f / 35.0f, -2.0f / 35.0f);
+    fs = __ffma2_rn(fs, delta, make_float2(2.0f / 15.0f, 2.0f / 15.0f));
+    fs = __ffma2_rn(fs, delta, make_float2(-1.0f / 3.0f, -1.0f / 3.0f));
+    fs = __ffma2_rn(fs, delta, make_float2(1.0f, 1.0f));
+    const float2 z = __fadd2_rn(__fadd2_rn(make_float2(1.0f, 1.0f), delta), t);
+    const float2 lg = make_float2(__logf(z.x), __logf(z.y));
+    const float2 fl = __fmul2_rn(lg, rs), ds = __fmul2_rn(t, fs);
+    const bool s0 = delta.x < 0.02f, s1 = delta.y < 0.02f;
+    const float2 f = make_float2(s0 ? fs.x : fl.x, s1 ? fs.y : fl.y);
+    const float2 d = make_float2(s0 ? ds.x : lg.x, s1 ? ds.y : lg.y);
+    const float2 u = __ffma2_rn(d, d, make_float2(1.0f, 1.0f));
+    w = make_float2(__fdividef(1.0f, u.x), __fdividef(1.0f, u.y));
+    rep = __fmul2_rn(w, __fmul2_rn(w, GF == 0 ? f : rs));
 }
 
 // Paired float32 arithmetic (one instruction for both components, each

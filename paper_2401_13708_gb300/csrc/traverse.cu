@@ -32,6 +32,10 @@ namespace hts {
 namespace {
 
 constexpr int kWalkBlock = 256;
+#ifndef LB
+#define LB 128
+#endif
+constexpr int kListBlock = LB;
 constexpr int kExactBlock = 64;
 
 // One node, read through the non-coherent path: a single 256-bit load (the
@@ -95,43 +99,73 @@ __device__ __forceinline__ void record_cost(const BlockOrder &bo, int b, long lo
         atomicAdd(&bo.cost[b], (unsigned)min((clock64() - t0) >> 6, 0xFFFFFll));
 }
 
-// Split walk (small problems, one embedding): the root is never accepted
-// (every point lies inside it, and r_cell / d >= 1 > theta), so each point's
-// walk is the union of its walks of the subtrees below a cut of the tree at
-// depth D.  One warp takes one 32-point chunk and one subtree of the cut (a
-// "frontier" entry): it first evaluates the criterion at the entry's
-// ancestors (depth 1 .. D-1) -- a lane that accepts one is done with this
+// Cuts of the tree (one embedding).  The root is never accepted (every point
+// lies inside it, and r_cell / d >= 1 > theta), so a walk is the union of the
+// walks of the subtrees below any cut of the tree.  A warp that takes one
+// 32-point chunk and one subtree first evaluates the criterion at the
+// subtree root's ancestors -- a lane that accepts one is done with this
 // subtree, and the interaction with that ancestor is counted by the first
-// frontier entry below it only -- then walks the subtree.  The partial sums
-// of the entries are added in entry order by walk_combine_kernel, so every
-// lane gets exactly the interactions of its full walk.
+// subtree below it only -- then walks the subtree: every lane gets exactly
+// the interactions of its full walk, in the same order.
+//   Sums:  a cut at depth D (walk_split_depth); one running sum per point and
+//          subtree, added in subtree order by walk_combine_kernel.
+//   Units: a finer cut (subtrees of at most about n / units points) that only
+//          divides the work of listing the interactions (list_f32_kernel).
 constexpr int kMaxSplitDepth = 3;
 constexpr int kMaxFrontier = 64;           // 4^3
 constexpr int64_t kSplitMaxN = 1 << 19;    // above: chunks alone fill the GPU (a cut measured slower at 1M)
 constexpr int64_t kSplitEntries = 1 << 22; // partial-sum buffer: entries x points
+constexpr int kMaxUnits = 256;
+constexpr int kMaxAnc = 8;                 // ancestors of a unit (deeper subtrees are not cut further)
 
-struct Frontier {
-    int node;                         // subtree root
-    int nanc;                         // ancestors below the root
-    int anc[kMaxSplitDepth];
-    int own;                          // bit k: this entry counts an accepted anc[k]
+struct Cut {
+    int node, end;     // subtree root and the index after the subtree
+    int nanc;          // ancestors below the root
+    int own;           // bit k: an accepted anc[k] is counted here
+    int anc[kMaxAnc];
+};
+
+struct CutTables {
+    Cut sums[kMaxFrontier];
+    Cut units[kMaxUnits];
+    int first[kMaxFrontier + 1];  // units of sum s: first[s] .. first[s + 1] - 1
+    int nsums, nunits;
 };
 
 struct SplitView {
-    const Frontier *fr;               // nullptr: no split
-    const int *count;                 // frontier entries
-    void *part;                       // [entry][n] partial sums (float4 / double4)
+    const CutTables *cut;             // nullptr: the whole tree is one subtree
+    void *part;                       // [sum][n] partial sums (float4 / double4); nullptr: one sum
 };
 
-struct NodesF {  // float32 nodes: cell test and skip index
+struct NodesF {  // float32 nodes: cell test, points and skip index
     const NodeF *nodes;
     __device__ bool cell(int k) const { return nodes[k].count >= 2.0f; }
+    __device__ int points(int k) const { return (int)nodes[k].count; }
     __device__ int skip(int k) const { return nodes[k].skip; }
 };
 struct NodesD {  // float64 nodes
     const NodeD *nodes;
     __device__ bool cell(int k) const { return nodes[k].count >= 2; }
+    __device__ int points(int k) const { return nodes[k].count; }
     __device__ int skip(int k) const { return nodes[k].skip; }
+};
+
+// Interaction lists between list_f32_kernel and sum_f32_kernel: pages of up
+// to 32 interactions (the node and the lanes of the chunk that take it).  The
+// first page of every (chunk, unit) has a fixed place; further ones come from
+// pools (chunk mod kListPools, so that the atomic counters are spread).  A
+// chunk whose pool runs out is flagged and walked directly by sum_f32_kernel.
+constexpr int kPage = 32;
+constexpr int kListPools = 256;
+
+struct ListView {
+    uint2 *entries;    // [page][kPage]: node, lane mask
+    int2 *head;        // per page: interactions held, next page (-1: none)
+    int *taken;        // per pool: pages taken
+    int *direct;       // per chunk: its pool ran out
+    int units;         // first pages per chunk
+    int chunks;
+    int per_pool;      // further pages per pool
 };
 
 // Per-lane state of the float32 walk: the query point (sorted position p),
@@ -141,6 +175,7 @@ struct LaneF {
     float2 qh, ql;  // position as hi / lo float pairs
     float twoil;
     int p;
+    int own;          // position of the point's own leaf (-1 in a bucket)
     float2 rxy, rsz;  // sums of k Delta and of (k s, mult w)
     int resume;
     unsigned long long c_acc, c_pair, c_crit;  // counting walk only
@@ -151,10 +186,10 @@ struct LaneF {
 // or one exact pair (mult = 1).
 // (The sums are paired: (rx, ry) += k Delta and (rs, z) += (k, mult) (s, w),
 // one fused multiply-add per pair, rounded as the scalar ones.)
-template <int GF>
+template <int GF, bool SMALL = false>
 __device__ __forceinline__ void add_pair_f32(LaneF &L, float2 d, float s, float delta, float mult, float il)
 {
-    const PairF t = pair_terms_f32<GF>(delta);
+    const PairF t = SMALL ? pair_terms_small_f32<GF>(delta) : pair_terms_f32<GF>(delta);
     const float k = mult * t.rep * il;
     L.rxy = __ffma2_rn(make_float2(k, k), d, L.rxy);
     L.rsz = __ffma2_rn(make_float2(k, mult), make_float2(s, t.w), L.rsz);
@@ -168,94 +203,269 @@ __device__ __forceinline__ float2 delta_f32(const LaneF &L, float2 h, float2 l, 
     return d;
 }
 
-// One visit of the warp's cursor at `node` (the node is the same for every
-// lane, so the branches on its kind are uniform).  Returns the next cursor:
-// at a cell, node + 1 if some open lane rejected it (the warp descends),
-// otherwise the index after its subtree; node + 1 after a leaf or bucket.
-// BOUNDED: a lane is open only below its own `end` (segments, split walk).
-template <int GF, bool COUNT, bool BOUNDED>
-__device__ __forceinline__ int visit_f32(int node, int end, LaneF &L, const NodeF *__restrict__ nodes,
-                                         const PointF *__restrict__ spts, int n)
+// Accepted interactions are collected first and evaluated later, a batch of
+// up to 32 at a time: lane e holds interaction e (the node and the lanes that
+// take it) until the batch is evaluated.  The cursor then never waits for a
+// pair term, and the pair terms of a batch are independent of each other and
+// of the walk.
+struct BatchF {
+    int node;       // interaction `lane`: its node
+    unsigned mask;  // and the lanes that take it
+    int count;      // interactions held (the same on every lane)
+};
+constexpr int kBatchFull = 28;  // evaluated above this (a trip of the walk adds up to four)
+
+// Node data of a batch, one array per field, so that the data of consecutive
+// interactions are register pairs of one (broadcast) shared-memory load.
+struct __align__(16) TileF {
+    float xh[32], yh[32], xl[32], yl[32], il[32], count[32];
+};
+
+// One visit of the warp's cursor at `node`: the lanes that accept the cell
+// (or take the leaf) are noted in the batch.  A leaf or bucket has threshold
+// -1, so every open lane takes it but the one whose own point it is (`own`:
+// the position of the lane's own leaf).  Returns the next cursor: node + 1 if
+// some open lane did not accept (the warp descends; past a leaf, node + 1 is
+// the index after it), otherwise the index after the node's subtree.
+// A lane is open from its `resume` to its own `end`.
+__device__ __forceinline__ int visit_f32(int node, int end, int lane, LaneF &L, BatchF &B,
+                                         const NodeF *__restrict__ nodes)
 {
     const NodeF c = load_node(nodes, node);
-    const bool open = node >= L.resume && (!BOUNDED || node < end);
-    int next = node + 1;
-    if (c.count >= 2) {  // cell: r_cell / d < theta  <=>  delta > thr
-        float s;
-        const float2 d = delta_f32(L, make_float2(c.xh, c.yh), make_float2(c.xl, c.yl), s);
-        const float delta = s * L.twoil * c.il;
-        const bool acc = open && delta > c.thr;
-        // the pair term runs on every lane when one accepts (no divergent
-        // branch); a lane that rejects adds it with weight 0, which leaves its
-        // sums unchanged (every term is finite: delta is clamped)
-        if (__any_sync(0xffffffffu, acc)) {
-            add_pair_f32<GF>(L, d, s, delta, acc ? c.count : 0.0f, c.il);
-            L.resume = acc ? c.skip : L.resume;
-        }
-        if (COUNT) {
-            L.c_crit += open ? 1 : 0;
-            L.c_acc += acc ? 1 : 0;
-        }
-        if (!__any_sync(0xffffffffu, open && !acc)) next = c.skip;
-    } else if (c.count == 1) {  // single-point leaf: the exact pair (not the lane's own point)
-        const bool take = open && __float_as_int(c.thr) != L.p;
-        if (__any_sync(0xffffffffu, take)) {  // as at a cell: weight 0 for the other lanes
-            float s;
-            const float2 d = delta_f32(L, make_float2(c.xh, c.yh), make_float2(c.xl, c.yl), s);
-            add_pair_f32<GF>(L, d, s, s * L.twoil * c.il, take ? 1.0f : 0.0f, c.il);
-            if (COUNT) L.c_pair += take ? 1 : 0;
-        }
-    } else {  // depth-29 bucket: each of its points exactly
-        const int lo = __float_as_int(c.thr), cnt = (int)(-c.count);
-        if (open && lo >= 0 && cnt > 0 && lo + cnt <= n) {
-            for (int k2 = 0; k2 < cnt; ++k2) {
-                if (lo + k2 == L.p) continue;
-                const PointF o = spts[lo + k2];
-                float s;
-                const float2 d = delta_f32(L, make_float2(o.xh, o.yh), make_float2(o.xl, o.yl), s);
-                add_pair_f32<GF>(L, d, s, s * L.twoil * o.il, 1.0f, o.il);
-                if (COUNT) ++L.c_pair;
-            }
-        }
+    float s;
+    delta_f32(L, make_float2(c.xh, c.yh), make_float2(c.xl, c.yl), s);
+    const float delta = s * L.twoil * c.il;
+    const bool open = node >= L.resume && node < end;
+    const bool acc = open && node != L.own && delta > c.thr;  // r_cell / d < theta  <=>  delta > thr
+    const unsigned m = __ballot_sync(0xffffffffu, acc);
+    const bool down = __any_sync(0xffffffffu, open && !acc);
+    if (acc) L.resume = c.skip;
+    if (lane == B.count) {
+        B.node = node;
+        B.mask = m;
     }
-    // next > node always: a cell's skip exceeds its position (emit writes no
-    // cell otherwise) and unwritten slots are zero (empty buckets)
-    return next;
+    B.count += m != 0u ? 1 : 0;
+    // next > node always: every node slot's skip exceeds its index
+    return down ? node + 1 : c.skip;
 }
 
-// One warp walks for the 32 sorted points of chunk `warp` (and, split, the
-// frontier entry `fi`).
-template <int GF, bool COUNT, bool SEG, bool SPLIT>
-__device__ __forceinline__ void walk_f32_chunk(int warp, int n, const NodeF *__restrict__ nodes,
-                                                const int *__restrict__ n_nodes, const PointF *__restrict__ spts,
-                                                const uint32_t *__restrict__ idx, double2 *frep, double *zi,
-                                                unsigned long long *counters, const SegView sv,
-                                                const SplitView sp, int fi)
+// The 32 x 32 bit matrix whose row `lane` is v, transposed: bit e of lane i's
+// result is bit i of lane e's v.
+__device__ __forceinline__ unsigned transpose_bits(unsigned v, int lane)
 {
-    const int lane = threadIdx.x & 31;
-    LaneF L;
-    L.p = warp * 32 + lane;
-    const bool valid = L.p < n;
-    {
-        const PointF q = spts[valid ? L.p : n - 1];
-        L.qh = make_float2(q.xh, q.yh);
-        L.ql = make_float2(q.xl, q.yl);
-        L.twoil = 2.0f * q.il;
+    unsigned m = 0x0000FFFFu;
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        const unsigned o = __shfl_xor_sync(0xffffffffu, v, j);
+        v = (lane & j) ? (v & ~m) | ((o >> j) & m) : (v & m) | ((o << j) & ~m);
+        m ^= m << (j >> 1);
     }
+    return v;
+}
+
+// Two consecutive interactions of a batch: k (the weight of Delta and s in the
+// sums) and w of both in paired FP32 arithmetic, each component rounded as the
+// scalar operations of add_pair_f32.
+template <int GF>
+__device__ __forceinline__ void two_terms_f32(const LaneF &L, float2 xh, float2 yh, float2 xl, float2 yl, float2 il,
+                                              float2 mult, float2 &k, float2 &w)
+{
+    const float2 dx = delta2(make_float2(L.qh.x, L.qh.x), make_float2(L.ql.x, L.ql.x), xh, xl);
+    const float2 dy = delta2(make_float2(L.qh.y, L.qh.y), make_float2(L.ql.y, L.ql.y), yh, yl);
+    const float2 s = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy));
+    float2 rep;
+    pair_terms2_f32<GF>(__fmul2_rn(__fmul2_rn(s, make_float2(L.twoil, L.twoil)), il), w, rep);
+    k = __fmul2_rn(__fmul2_rn(mult, rep), il);
+}
+
+// A depth-29 bucket: each of its points exactly (not the lane's own).
+template <int GF, bool COUNT>
+__device__ __forceinline__ void add_bucket_f32(LaneF &L, const NodeF &c, const PointF *__restrict__ spts, int n)
+{
+    const int lo = __float_as_int(c.il), cnt = (int)(-c.count);
+    if (lo < 0 || cnt <= 0 || lo + cnt > n) return;
+    for (int k = 0; k < cnt; ++k) {
+        if (lo + k == L.p) continue;
+        const PointF o = spts[lo + k];
+        float s;
+        const float2 d = delta_f32(L, make_float2(o.xh, o.yh), make_float2(o.xl, o.yl), s);
+        add_pair_f32<GF>(L, d, s, s * L.twoil * o.il, 1.0f, o.il);
+        if (COUNT) ++L.c_pair;
+    }
+}
+
+// A batch that holds a bucket: interaction by interaction.
+template <int GF>
+__device__ __forceinline__ void add_with_buckets_f32(LaneF &L, int bnode, unsigned bmask, int count, int lane,
+                                                     const NodeF *__restrict__ nodes,
+                                                     const PointF *__restrict__ spts, int n)
+{
+    for (int e = 0; e < count; ++e) {
+        const NodeF c = load_node(nodes, __shfl_sync(0xffffffffu, bnode, e));
+        const bool take = (__shfl_sync(0xffffffffu, bmask, e) >> lane) & 1u;
+        if (!take) continue;
+        if (c.count < 0.0f) {
+            add_bucket_f32<GF, false>(L, c, spts, n);
+            continue;
+        }
+        float s;
+        const float2 d = delta_f32(L, make_float2(c.xh, c.yh), make_float2(c.xl, c.yl), s);
+        add_pair_f32<GF>(L, d, s, s * L.twoil * c.il, c.count, c.il);
+    }
+}
+
+// The point of lane `lane` of a chunk (the last point again past the end).
+__device__ __forceinline__ void load_lane(LaneF &L, int chunk, int lane, int n, const PointF *__restrict__ spts,
+                                          const int *__restrict__ leaf)
+{
+    L.p = chunk * 32 + lane;
+    const int k = min(L.p, n - 1);
+    const PointF q = spts[k];
+    L.qh = make_float2(q.xh, q.yh);
+    L.ql = make_float2(q.xl, q.yl);
+    L.twoil = 2.0f * q.il;
+    L.own = leaf[k];
     L.rxy = L.rsz = make_float2(0.f, 0.f);
     L.c_acc = L.c_pair = L.c_crit = 0;
+}
+
+// The ancestors of a cut's subtree: a lane that accepts one is done (returns
+// false); the interaction goes to the batch if it is counted here.
+__device__ __forceinline__ bool visit_ancestors_f32(const Cut &F, bool live, int lane, LaneF &L, BatchF &B,
+                                                    const NodeF *__restrict__ nodes)
+{
+    const int na = F.nanc, owned = F.own;
+    for (int k = 0; k < na; ++k) {
+        const int at = F.anc[k];
+        const NodeF a = load_node(nodes, at);
+        const bool own = (owned >> k) & 1;
+        float s;
+        delta_f32(L, make_float2(a.xh, a.yh), make_float2(a.xl, a.yl), s);
+        const bool acc = live && s * L.twoil * a.il > a.thr;
+        const unsigned m = __ballot_sync(0xffffffffu, acc && own);
+        if (lane == B.count) {
+            B.node = at;
+            B.mask = m;
+        }
+        B.count += m != 0u ? 1 : 0;
+        live = live && !acc;
+    }
+    return live;
+}
+
+// A chunk's sums into its points' results (or, split, into the partial sums
+// of subtree `sum`).
+__device__ __forceinline__ void store_lane(const LaneF &L, int sum, int n, const uint32_t *__restrict__ idx,
+                                           double2 *frep, double *zi, void *part)
+{
+    if (L.p >= n) return;
+    if (part) {
+        reinterpret_cast<float4 *>(part)[(size_t)sum * n + L.p] = make_float4(L.rxy.x, L.rxy.y, L.rsz.x, L.rsz.y);
+        return;
+    }
+    const uint32_t i = idx[L.p];
+    double x = (double)L.qh.x + (double)L.ql.x, y = (double)L.qh.y + (double)L.ql.y;
+    double il = 0.5 * (double)L.twoil;
+    double rsd = il * (double)L.rsz.x;
+    frep[i] = make_double2(4.0 * il * ((double)L.rxy.x + rsd * x), 4.0 * il * ((double)L.rxy.y + rsd * y));
+    zi[i] = (double)L.rsz.y;
+}
+
+// One visit of the direct walk's cursor at `node`, whose data `c` are loaded:
+// as visit_f32, but the pair term is added at once.  The next node's load is
+// issued before it, so that the load's latency and the pair term's overlap:
+// a walk of one wave of blocks lasts as long as its longest chunk's chain of
+// visits (load, criterion, vote, pair term, next load), and the overlap cut a
+// visit from ~420 to ~290 cycles (walk at N = 70,000: 520 -> 367 us; N =
+// 131,071, theta = 0.2: 6.2 -> 4.4 ms).  At N = 1M, several waves, issue slots
+// bound the walk (88% of them taken, counting the second slot of a paired
+// FP32 instruction) and the overlap changes nothing.  Leaves take the cells'
+// path (threshold -1), so a visit tests the kind of node only for buckets.
+// The term runs on every lane when one takes it (no divergent branch); a lane
+// that does not adds it with weight 0, which leaves its sums unchanged (every
+// term is finite: delta is clamped).
+template <int GF, bool COUNT, bool BOUNDED, bool SMALL>
+__device__ __forceinline__ void visit_direct_f32(int &node, NodeF &c, int end, LaneF &L,
+                                                 const NodeF *__restrict__ nodes, const PointF *__restrict__ spts,
+                                                 int n)
+{
+    float s;
+    const float2 d = delta_f32(L, make_float2(c.xh, c.yh), make_float2(c.xl, c.yl), s);
+    const float delta = s * L.twoil * c.il;
+    const bool open = node >= L.resume && (!BOUNDED || node < end);
+    const bool acc = open && node != L.own && delta > c.thr;
+    const bool some = __any_sync(0xffffffffu, acc), down = __any_sync(0xffffffffu, open && !acc);
+    node = down ? node + 1 : c.skip;
+    const NodeF next = load_node(nodes, node);
+    if (COUNT) {
+        L.c_crit += open && c.count >= 2.0f ? 1 : 0;
+        L.c_acc += acc && c.count >= 2.0f ? 1 : 0;
+        L.c_pair += acc && c.count == 1.0f ? 1 : 0;
+    }
+    if (some) {
+        L.resume = acc ? c.skip : L.resume;
+        if (c.count >= 0.0f)
+            add_pair_f32<GF, SMALL>(L, d, s, delta, acc ? c.count : 0.0f, c.il);
+        else if (acc)
+            add_bucket_f32<GF, COUNT>(L, c, spts, n);
+    }
+    c = next;
+}
+
+// Largest disk radius of each segment's points (the root annulus of its tree).
+struct AnnulusView {
+    const unsigned long long *bounds;  // [2s + 1]: largest split coordinate of segment s (float64 bits)
+    const uint64_t *keys;              // sorted keys (segment id in the top bits); nullptr: one segment
+    int rule, last;                    // split rule; last sorted position
+};
+
+// Whether every delta of the warp's points is below the series limit of
+// pair_terms_f32, by the radii alone: |y_i - c| <= |y_i| + R and il_c <=
+// 1 / (1 - R^2) for every point and midpoint c of a tree whose points lie
+// within radius R (a midpoint lies in the hull of its points).  The same on
+// every lane; a warp that straddles segments takes the larger R for all lanes,
+// so that the terms of lanes that are not open stay finite too.
+__device__ __forceinline__ bool all_small(const LaneF &L, int lane, const AnnulusView &an)
+{
+    const int p0 = __shfl_sync(0xffffffffu, L.p, 0);
+    const int s = an.keys ? (int)(an.keys[p0 + min(lane, an.last - p0)] >> kSegShift) : 0;
+    const float v = (float)__longlong_as_double((long long)an.bounds[2 * s + 1]);
+    const float R2 = an.rule == HTS_EQUAL_AREA ? (v - 1.0f) / (v + 1.0f) : v * v;
+    const float R = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sqrtf(fmaxf(R2, 0.0f)))));
+    const float r = sqrtf(L.qh.x * L.qh.x + L.qh.y * L.qh.y) + R;
+    // (1% below the limit: far more than the roundings above)
+    return __all_sync(0xffffffffu, R < 0.5f && r * r * L.twoil < 0.0198f * (1.0f - R * R));
+}
+
+// One warp walks for a chunk (sum `sum` of the cut when there are partial
+// sums).  kWalkTrip visits per trip and one test of the cursor: the loop-back
+// branch and the cursor tests cost (8 visits per trip against 4, walk at
+// N = 131,071, theta = 0.2: 4.57 against 4.78 ms; at N = 1M, spread: 6.11
+// against 6.32).  The cursor may run up to kWalkTrip - 1 nodes past `stop`
+// (and the load one further): past the last node the tree build leaves empty
+// slots (visited as no-ops), and below it every lane's own bound `end` closes
+// it (BOUNDED).
+// The first iterations, while the embedding is within a radius of ~0.05, take
+// the loop without the logarithm (all_small; walk at N = 1M from Y0: 2.58 ->
+// 2.30 ms, 64 embeddings: 0.74 -> 0.65 ms).
+template <int GF, bool COUNT, bool SEG, bool SPLIT>
+__device__ __forceinline__ void walk_f32_chunk(LaneF &L, int n, int lane, const NodeF *__restrict__ nodes,
+                                                const int *__restrict__ n_nodes, const PointF *__restrict__ spts,
+                                                unsigned long long *counters, const SegView sv, const CutTables *cut,
+                                                int sum, const AnnulusView &an)
+{
+    const bool valid = L.p < n;
     unsigned long long c_visit = 0;
     const int m = min(*n_nodes, 2 * n);
     int root = 0, end = m;
     if (SEG) segment_range(sv, valid ? L.p : n - 1, m, root, end);
     bool live = valid;
-    if (SPLIT) {  // frontier entry: ancestors first, then the subtree [node, skip)
-        const Frontier F = sp.fr[fi];
-#pragma unroll
-        for (int k = 0; k < kMaxSplitDepth; ++k) {
-            if (k >= F.nanc) break;
+    if (SPLIT) {  // ancestors first, then the subtree [node, end)
+        const Cut &F = cut->sums[sum];
+        const int na = F.nanc, owned = F.own;
+        for (int k = 0; k < na; ++k) {
             const NodeF a = load_node(nodes, F.anc[k]);
-            const bool own = (F.own >> k) & 1;
+            const bool own = (owned >> k) & 1;
             float s;
             const float2 d = delta_f32(L, make_float2(a.xh, a.yh), make_float2(a.xl, a.yl), s);
             const float delta = s * L.twoil * a.il;
@@ -269,36 +479,26 @@ __device__ __forceinline__ void walk_f32_chunk(int warp, int n, const NodeF *__r
             }
         }
         root = F.node;
-        end = min(load_node(nodes, F.node).skip, m);
+        end = F.end;
     }
     L.resume = live ? root : INT_MAX;
     int node = SEG ? __shfl_sync(0xffffffffu, root, 0) : root;  // lane 0 holds the first segment
     const int stop = SEG ? __reduce_max_sync(0xffffffffu, valid ? end : 0) : end;
-    // four visits per trip and one test of the cursor: in this issue-bound
-    // loop the loop-back branch and the cursor tests cost.  The cursor may run
-    // up to three nodes past `stop`: past the last node the tree build leaves
-    // four empty slots (visited as no-ops), and below it every lane's own
-    // bound `end` closes it (BOUNDED).
-    constexpr bool kBounded = SEG || SPLIT;
-    while (node < stop) {
-        if (COUNT && lane == 0) ++c_visit;  // (counted: visits below stop)
-        node = visit_f32<GF, COUNT, kBounded>(node, end, L, nodes, spts, n);
-        if (COUNT && lane == 0 && node < stop) ++c_visit;
-        node = visit_f32<GF, COUNT, kBounded>(node, end, L, nodes, spts, n);
-        if (COUNT && lane == 0 && node < stop) ++c_visit;
-        node = visit_f32<GF, COUNT, kBounded>(node, end, L, nodes, spts, n);
-        if (COUNT && lane == 0 && node < stop) ++c_visit;
-        node = visit_f32<GF, COUNT, kBounded>(node, end, L, nodes, spts, n);
+    NodeF c = load_node(nodes, node);
+    if (!COUNT && all_small(L, lane, an)) {
+        while (node < stop) {
+#pragma unroll
+            for (int k = 0; k < kWalkTrip; ++k)
+                visit_direct_f32<GF, false, SEG || SPLIT, true>(node, c, end, L, nodes, spts, n);
+        }
+        return;
     }
-    if (SPLIT && valid) {
-        reinterpret_cast<float4 *>(sp.part)[(size_t)fi * n + L.p] = make_float4(L.rxy.x, L.rxy.y, L.rsz.x, L.rsz.y);
-    } else if (valid) {
-        const uint32_t i = idx[L.p];
-        double x = (double)L.qh.x + (double)L.ql.x, y = (double)L.qh.y + (double)L.ql.y;
-        double il = 0.5 * (double)L.twoil;
-        double rsd = il * (double)L.rsz.x;
-        frep[i] = make_double2(4.0 * il * ((double)L.rxy.x + rsd * x), 4.0 * il * ((double)L.rxy.y + rsd * y));
-        zi[i] = (double)L.rsz.y;
+    while (node < stop) {
+#pragma unroll
+        for (int k = 0; k < kWalkTrip; ++k) {
+            if (COUNT && lane == 0 && node < stop) ++c_visit;  // (counted: visits below stop)
+            visit_direct_f32<GF, COUNT, SEG || SPLIT, false>(node, c, end, L, nodes, spts, n);
+        }
     }
     if (COUNT) {
         unsigned long long c_acc = L.c_acc, c_pair = L.c_pair, c_crit = L.c_crit;
@@ -311,32 +511,249 @@ __device__ __forceinline__ void walk_f32_chunk(int warp, int n, const NodeF *__r
             atomicAdd(&counters[0], c_acc);
             atomicAdd(&counters[1], c_pair);
             atomicAdd(&counters[2], c_visit);
-            atomicAdd(&counters[3], (unsigned long long)min(32, n - warp * 32));
+            atomicAdd(&counters[3], (unsigned long long)min(32, n - L.p));
             atomicAdd(&counters[4], c_crit);
         }
     }
 }
 
-// One warp per chunk of 32 sorted points; the warps of a block (blockDim.x /
-// 32 <= kWalkBlock / 32, picked by the autotuner) take consecutive chunks, so
-// their walks share node data in L1.  The block size does not change results.
+// Direct walk: one warp per chunk of 32 sorted points (and, split, per sum:
+// grid.y); the warps of a block (blockDim.x / 32 <= kWalkBlock / 32, picked by
+// the autotuner) take consecutive chunks, so their walks share node data in
+// L1.  The block size does not change results.
 template <int GF, bool COUNT, bool SEG, bool SPLIT>
-__global__ void __launch_bounds__(kWalkBlock) walk_f32_kernel(int n, const NodesF nodes,
+__global__ void __launch_bounds__(kWalkBlock) walk_f32_kernel(int n, const NodeF *__restrict__ nodes,
                                                               const int *__restrict__ n_nodes,
                                                               const PointF *__restrict__ spts,
+                                                              const int *__restrict__ leaf,
                                                               const uint32_t *__restrict__ idx, double2 *frep,
                                                               double *zi, unsigned long long *counters,
-                                                              const SegView sv, const SplitView sp,
+                                                              const SegView sv, const SplitView sp, const AnnulusView an,
                                                               const BlockOrder bo)
 {
     const int b = logical_block(bo);
-    const int warp = (b * blockDim.x + threadIdx.x) >> 5;
-    if (warp * 32 >= n) return;
-    if (SPLIT && (int)blockIdx.y >= *sp.count) return;
+    const int chunk = (b * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (chunk * 32 >= n) return;
+    if (SPLIT && (int)blockIdx.y >= sp.cut->nsums) return;
     const long long t0 = clock64();
-    walk_f32_chunk<GF, COUNT, SEG, SPLIT>(warp, n, nodes.nodes, n_nodes, spts, idx, frep, zi, counters, sv, sp,
-                                          blockIdx.y);
+    LaneF L;
+    load_lane(L, chunk, lane, n, spts, leaf);
+    walk_f32_chunk<GF, COUNT, SEG, SPLIT>(L, n, lane, nodes, n_nodes, spts, counters, sv, sp.cut, blockIdx.y, an);
+    store_lane(L, blockIdx.y, n, idx, frep, zi, SPLIT ? sp.part : nullptr);
     record_cost(bo, b, t0);
+}
+
+// Lists the interactions of a chunk (grid.x: chunks, a warp each; the warps of
+// a block take consecutive chunks, so their walks share node data in L1) with
+// one unit of the tree (grid.y).
+__global__ void __launch_bounds__(kListBlock, 6) list_f32_kernel(int n, const NodeF *__restrict__ nodes,
+                                                                 const PointF *__restrict__ spts,
+                                                                 const int *__restrict__ leaf,
+                                                                 const CutTables *__restrict__ cut, const ListView lv)
+{
+    const int chunk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (chunk >= lv.chunks || (int)blockIdx.y >= cut->nunits) return;
+    LaneF L;
+    load_lane(L, chunk, lane, n, spts, leaf);
+    BatchF B;
+    B.node = 0;
+    B.mask = 0u;
+    B.count = 0;
+    const Cut &F = cut->units[blockIdx.y];
+    const bool live = visit_ancestors_f32(F, L.p < n, lane, L, B, nodes);
+    int node = F.node;
+    const int end = F.end;
+    L.resume = live ? node : INT_MAX;
+    if (!__any_sync(0xffffffffu, live)) node = end;
+    int page = chunk * lv.units + (int)blockIdx.y;
+    const int pool = chunk & (kListPools - 1);
+    while (node < end) {  // (a page holds what a trip can add to kBatchFull)
+#pragma unroll
+        for (int k = 0; k < kPage - kBatchFull; ++k) node = visit_f32(node, end, lane, L, B, nodes);
+        if (B.count > kBatchFull) {  // the page is full: write it, take another
+            if (lane < B.count) lv.entries[(size_t)page * kPage + lane] = make_uint2((unsigned)B.node, B.mask);
+            int next = 0;
+            if (lane == 0) {
+                next = atomicAdd(&lv.taken[pool], 1);
+                next = next < lv.per_pool ? lv.chunks * lv.units + pool * lv.per_pool + next : -1;
+                lv.head[page] = make_int2(B.count, next);
+                if (next < 0) lv.direct[chunk] = 1;
+            }
+            next = __shfl_sync(0xffffffffu, next, 0);
+            if (next < 0) return;
+            page = next;
+            B.count = 0;
+        }
+    }
+    if (lane < B.count) lv.entries[(size_t)page * kPage + lane] = make_uint2((unsigned)B.node, B.mask);
+    if (lane == 0) lv.head[page] = make_int2(B.count, -1);
+}
+
+// A block evaluates the listed interactions of a chunk (grid.x; grid.y: the
+// sum).  The interactions of consecutive pages make batches of up to 32, dealt
+// to the block's kSumWarps warps in turn: the pair terms of different batches
+// run beside each other, and only the running sums go from warp to warp in
+// batch order, so every sum is taken in the order of the walk.  With one warp
+// per chunk the longest chunk takes most of the kernel (N = 20,011, 2,500
+// (chunk, sum) pairs: 180 us with one warp each, 133 us with four).
+constexpr int kSumWarps = 4;
+
+struct SumShared {
+    TileF tile[kSumWarps];
+    float2 term[kSumWarps][32][32];  // [warp][interaction][lane]: k, w (0 where the lane does not take it)
+    float4 sums[32];                 // running sums of the lanes' points after the last finished batch
+};
+
+// Waits for / passes on the running sums: barrier 1 + w pairs the warp w that
+// waits with the warp before it.
+__device__ __forceinline__ void sums_wait(int w)
+{
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + w) : "memory");
+}
+__device__ __forceinline__ void sums_pass(int w)
+{
+    __threadfence_block();
+    asm volatile("bar.arrive %0, 64;" ::"r"(1 + (w + 1 == kSumWarps ? 0 : w + 1)) : "memory");
+}
+
+// One batch of a warp (its `batch`-th in the block's order): terms, then, in
+// turn, the sums.
+template <int GF>
+__device__ __forceinline__ void sum_batch_f32(LaneF &L, const BatchF &B, int batch, int w, int lane, SumShared &S,
+                                              const NodeF *__restrict__ nodes, const PointF *__restrict__ spts, int n)
+{
+    TileF &T = S.tile[w];
+    const bool have = lane < B.count;
+    const unsigned mask = have ? B.mask : 0u;
+    const NodeF c = load_node(nodes, have ? B.node : 0);
+    const bool bucket = __any_sync(0xffffffffu, have && c.count < 0.0f);
+    if (!bucket) {
+        __syncwarp();  // the warp's previous batch has been read
+        T.xh[lane] = c.xh;
+        T.yh[lane] = c.yh;
+        T.xl[lane] = c.xl;
+        T.yl[lane] = c.yl;
+        T.il[lane] = c.il;
+        T.count[lane] = c.count;
+        unsigned bits = transpose_bits(mask, lane);
+        __syncwarp();
+        for (int e = 0; e < B.count; e += 4) {  // (slots past the count: no lane takes them)
+            const float4 xh = *reinterpret_cast<const float4 *>(&T.xh[e]), yh = *reinterpret_cast<const float4 *>(&T.yh[e]);
+            const float4 xl = *reinterpret_cast<const float4 *>(&T.xl[e]), yl = *reinterpret_cast<const float4 *>(&T.yl[e]);
+            const float4 il = *reinterpret_cast<const float4 *>(&T.il[e]);
+            const float4 ct = *reinterpret_cast<const float4 *>(&T.count[e]);
+            const bool t0 = bits & 1u, t1 = bits & 2u, t2 = bits & 4u, t3 = bits & 8u;
+            float2 k, v;
+            two_terms_f32<GF>(L, make_float2(xh.x, xh.y), make_float2(yh.x, yh.y), make_float2(xl.x, xl.y),
+                              make_float2(yl.x, yl.y), make_float2(il.x, il.y),
+                              make_float2(t0 ? ct.x : 0.0f, t1 ? ct.y : 0.0f), k, v);
+            S.term[w][e][lane] = make_float2(k.x, t0 ? v.x : 0.0f);
+            S.term[w][e + 1][lane] = make_float2(k.y, t1 ? v.y : 0.0f);
+            two_terms_f32<GF>(L, make_float2(xh.z, xh.w), make_float2(yh.z, yh.w), make_float2(xl.z, xl.w),
+                              make_float2(yl.z, yl.w), make_float2(il.z, il.w),
+                              make_float2(t2 ? ct.z : 0.0f, t3 ? ct.w : 0.0f), k, v);
+            S.term[w][e + 2][lane] = make_float2(k.x, t2 ? v.x : 0.0f);
+            S.term[w][e + 3][lane] = make_float2(k.y, t3 ? v.y : 0.0f);
+            bits >>= 4;
+        }
+    }
+    if (batch > 0) {
+        sums_wait(w);
+        const float4 r = S.sums[lane];
+        L.rxy = make_float2(r.x, r.y);
+        L.rsz = make_float2(r.z, r.w);
+    }
+    if (!bucket) {
+        for (int e = 0; e < B.count; e += 4) {
+            const float4 xh = *reinterpret_cast<const float4 *>(&T.xh[e]), yh = *reinterpret_cast<const float4 *>(&T.yh[e]);
+            const float4 xl = *reinterpret_cast<const float4 *>(&T.xl[e]), yl = *reinterpret_cast<const float4 *>(&T.yl[e]);
+            const float4 ct = *reinterpret_cast<const float4 *>(&T.count[e]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 t = S.term[w][e + q][lane];
+                float s;
+                const float2 d = delta_f32(L, make_float2((&xh.x)[q], (&yh.x)[q]), make_float2((&xl.x)[q], (&yl.x)[q]), s);
+                L.rxy = __ffma2_rn(make_float2(t.x, t.x), d, L.rxy);
+                L.rsz = __ffma2_rn(make_float2(t.x, (&ct.x)[q]), make_float2(s, t.y), L.rsz);
+            }
+        }
+    } else {
+        add_with_buckets_f32<GF>(L, B.node, mask, B.count, lane, nodes, spts, n);
+        __syncwarp();
+    }
+    S.sums[lane] = make_float4(L.rxy.x, L.rxy.y, L.rsz.x, L.rsz.y);
+    sums_pass(w);
+}
+
+template <int GF, bool SPLIT>
+__global__ void __launch_bounds__(32 * kSumWarps, 6) sum_f32_kernel(int n, const NodeF *__restrict__ nodes,
+                                                                    const int *__restrict__ n_nodes,
+                                                                    const PointF *__restrict__ spts,
+                                                                    const int *__restrict__ leaf,
+                                                                    const uint32_t *__restrict__ idx, double2 *frep,
+                                                                    double *zi, const SplitView sp, const ListView lv,
+                                                                    const AnnulusView an)
+{
+    __shared__ SumShared S;
+    const int chunk = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int sum = SPLIT ? (int)blockIdx.y : 0;
+    if (sum >= sp.cut->nsums) return;
+    LaneF L;
+    load_lane(L, chunk, lane, n, spts, leaf);
+    if (lv.direct[chunk]) {
+        if (w > 0) return;
+        walk_f32_chunk<GF, false, false, SPLIT>(L, n, lane, nodes, n_nodes, spts, nullptr, SegView{}, sp.cut, sum, an);
+        store_lane(L, sum, n, idx, frep, zi, SPLIT ? sp.part : nullptr);
+        return;
+    }
+    BatchF B;
+    B.node = 0;
+    B.mask = 0u;
+    B.count = 0;
+    int batch = 0, turn = 0;  // the batch being gathered, and its warp: batch mod kSumWarps
+    const int u0 = sp.cut->first[sum], u1 = sp.cut->first[sum + 1];
+    for (int ub = u0; ub < u1; ub += 32) {
+        const int2 h = ub + lane < u1 ? lv.head[chunk * lv.units + ub + lane] : make_int2(0, -1);
+        unsigned todo = __ballot_sync(0xffffffffu, h.x > 0);
+        while (todo) {
+            const int j = __ffs((int)todo) - 1;
+            todo &= todo - 1;
+            int page = chunk * lv.units + ub + j;
+            int count = __shfl_sync(0xffffffffu, h.x, j), next = __shfl_sync(0xffffffffu, h.y, j);
+            while (true) {
+                if (B.count + count > 32) {
+                    if (turn == w) sum_batch_f32<GF>(L, B, batch, w, lane, S, nodes, spts, n);
+                    ++batch;
+                    turn = turn + 1 == kSumWarps ? 0 : turn + 1;
+                    B.count = 0;
+                }
+                if (turn == w && lane >= B.count && lane < B.count + count) {
+                    const uint2 e = lv.entries[(size_t)page * kPage + lane - B.count];
+                    B.node = (int)e.x;
+                    B.mask = e.y;
+                }
+                B.count += count;
+                if (next < 0) break;
+                page = next;
+                const int2 g = lv.head[page];
+                count = g.x;
+                next = g.y;
+            }
+        }
+    }
+    if (B.count > 0) {
+        if (turn == w) sum_batch_f32<GF>(L, B, batch, w, lane, S, nodes, spts, n);
+        ++batch;
+        turn = turn + 1 == kSumWarps ? 0 : turn + 1;
+    }
+    if (turn != w) return;
+    if (batch > 0) {  // the warp after the last batch's takes the sums
+        sums_wait(w);
+        const float4 r = S.sums[lane];
+        L.rxy = make_float2(r.x, r.y);
+        L.rsz = make_float2(r.z, r.w);
+    }
+    store_lane(L, sum, n, idx, frep, zi, SPLIT ? sp.part : nullptr);
 }
 
 template <int GF, bool COUNT, bool SEG, bool SPLIT>
@@ -359,10 +776,8 @@ __device__ __forceinline__ void walk_f64_chunk(int warp, int n, const NodeD *__r
     unsigned long long c_acc = 0, c_pair = 0, c_visit = 0;
     bool live = valid;
     if (SPLIT) {  // as in the float32 walk
-        const Frontier F = sp.fr[fi];
-#pragma unroll
-        for (int k = 0; k < kMaxSplitDepth; ++k) {
-            if (k >= F.nanc) break;
+        const Cut &F = sp.cut->sums[fi];
+        for (int k = 0; k < F.nanc; ++k) {
             const NodeD a = nodes[F.anc[k]];
             double dx = q.x - a.x, dy = q.y - a.y;
             double s = fma(dx, dx, dy * dy);
@@ -382,7 +797,7 @@ __device__ __forceinline__ void walk_f64_chunk(int warp, int n, const NodeD *__r
             }
         }
         root = F.node;
-        end = min(nodes[F.node].skip, m);
+        end = F.end;
     }
     int resume = live ? root : INT_MAX;
     int node = SEG ? __shfl_sync(0xffffffffu, root, 0) : root;
@@ -468,6 +883,7 @@ template <int GF, bool COUNT, bool SEG, bool SPLIT>
 __global__ void __launch_bounds__(kWalkBlock) walk_f64_kernel(int n, const NodeD *__restrict__ nodes,
                                                               const int *__restrict__ n_nodes,
                                                               const PointD *__restrict__ spts,
+                                                              const int *__restrict__ leaf,
                                                               const uint32_t *__restrict__ idx, double2 *frep,
                                                               double *zi, unsigned long long *counters,
                                                               const SegView sv, const SplitView sp,
@@ -476,7 +892,7 @@ __global__ void __launch_bounds__(kWalkBlock) walk_f64_kernel(int n, const NodeD
     const int b = logical_block(bo);
     const int warp = (b * blockDim.x + threadIdx.x) >> 5;
     if (warp * 32 >= n) return;
-    if (SPLIT && (int)blockIdx.y >= *sp.count) return;
+    if (SPLIT && (int)blockIdx.y >= sp.cut->nsums) return;
     const long long t0 = clock64();
     walk_f64_chunk<GF, COUNT, SEG, SPLIT>(warp, n, nodes, n_nodes, spts, idx, frep, zi, counters, sv, sp, blockIdx.y);
     record_cost(bo, b, t0);
@@ -519,80 +935,141 @@ __global__ void __launch_bounds__(1024) walk_order_kernel(unsigned *cost, int nb
     if (threadIdx.x == 0) order[0] = nb;
 }
 
-// The frontier of the cut at `depth` (single thread; at most 4^depth entries
-// in pre-order).  A cell with more than 4 children or a skip that does not
-// advance is a broken tree: status bit 2, no entries (the walk then does no
-// work and the error is reported).
+// Both cuts (one block): level by level from the root, one thread per subtree,
+// every cell above `depth` into its children, then every cell of more than
+// `grain` points, while the subtrees fit `cap`; in pre-order throughout.  A
+// cell with more than 4 children or a skip that does not advance is a broken
+// tree: status bit 2, no subtrees (the walk then does no work and the error is
+// reported).
 template <typename NV>
-__global__ void frontier_kernel(const NV nodes, const int *__restrict__ n_nodes, int n, int depth, Frontier *fr,
-                                int *count, int *status)
+__global__ void __launch_bounds__(kMaxUnits) cut_kernel(const NV nodes, const int *__restrict__ n_nodes, int n,
+                                                        int depth, int grain, int cap, CutTables *ct, int *status)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ Cut sub[2][kMaxUnits];
+    __shared__ int sum_of[2][kMaxUnits];
+    __shared__ int wtot[kMaxUnits / 32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int m = min(*n_nodes, 2 * n);
-    Frontier a[kMaxFrontier], b[kMaxFrontier];
-    int na = 1;
-    a[0].node = 0;
-    a[0].nanc = 0;
-    a[0].own = 0;
-    bool bad = m <= 0;
-    for (int d = 0; d < depth && !bad; ++d) {
-        int nb = 0;
-        for (int e = 0; e < na && !bad; ++e) {
-            const Frontier &E = a[e];
-            if (!nodes.cell(E.node)) {  // leaf or bucket: stays an entry
-                if (nb >= kMaxFrontier) { bad = true; break; }
-                b[nb++] = E;
-                continue;
-            }
-            const int cskip = nodes.skip(E.node);
-            bool first = true;
-            int kids = 0;
-            for (int ch = E.node + 1; ch < cskip && ch < m;) {
-                if (++kids > 4 || nb >= kMaxFrontier) { bad = true; break; }
-                Frontier F = E;
-                F.node = ch;
-                F.own = first ? E.own : 0;
-                if (d >= 1) {  // E is below the root: an ancestor of its children
-                    F.anc[F.nanc] = E.node;
-                    if (first) F.own |= 1 << F.nanc;
-                    F.nanc += 1;
+    int cur = 0, count = 1, nsums = 1;
+    if (t == 0) {
+        sub[0][0] = Cut{0, m, 0, 0, {0, 0, 0, 0, 0, 0, 0, 0}};
+        sum_of[0][0] = 0;
+    }
+    __syncthreads();
+    int bad = m <= 0 ? 1 : 0;
+    for (int lev = 0; lev < depth + kMaxAnc && !bad; ++lev) {
+        Cut U;
+        int kids = 0, ch[4] = {0, 0, 0, 0};
+        bool expand = false;
+        if (t < count) {
+            U = sub[cur][t];
+            expand = nodes.cell(U.node) && (lev < depth || (nodes.points(U.node) > grain && U.nanc < kMaxAnc));
+            kids = expand ? 0 : 1;
+            if (expand) {
+                for (int c = U.node + 1; c < U.end && !bad;) {
+                    const int nx = nodes.skip(c);
+                    if (kids == 4 || nx <= c) {
+                        bad = 1;
+                        break;
+                    }
+                    ch[kids++] = c;
+                    c = nx;
                 }
-                b[nb++] = F;
-                first = false;
-                const int nx = nodes.skip(ch);
-                if (nx <= ch) { bad = true; break; }
-                ch = nx;
             }
         }
-        for (int e = 0; e < nb; ++e) a[e] = b[e];
-        na = nb;
+        int incl = kids;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) wtot[w] = incl;
+        bad = __syncthreads_or(bad);
+        const int grown = __syncthreads_or(expand ? 1 : 0);
+        int at = incl - kids, total = 0;
+        for (int k = 0; k < kMaxUnits / 32; ++k) {
+            if (k < w) at += wtot[k];
+            total += wtot[k];
+        }
+        if (bad || (lev >= depth && !grown) || total > cap) {
+            bad |= lev < depth && total > cap ? 1 : 0;
+            break;
+        }
+        if (t < count) {
+            const int s = sum_of[cur][t];
+            if (!expand) {
+                sub[cur ^ 1][at] = U;
+                sum_of[cur ^ 1][at] = s;
+            } else {
+                const int na = U.nanc;
+                const bool below = U.node != 0;  // an ancestor of its children, unless it is the root
+                for (int k = 0; k < kids; ++k) {
+                    Cut F = U;
+                    F.node = ch[k];
+                    F.end = k + 1 < kids ? ch[k + 1] : U.end;
+                    F.own = k == 0 ? U.own | (below ? 1 << na : 0) : 0;
+                    if (below) {
+                        for (int q = 0; q < kMaxAnc; ++q)
+                            if (q == na) F.anc[q] = U.node;
+                        F.nanc = na + 1;
+                    }
+                    sub[cur ^ 1][at + k] = F;
+                    sum_of[cur ^ 1][at + k] = s;
+                }
+            }
+        }
+        __syncthreads();
+        cur ^= 1;
+        count = total;
+        if (lev + 1 == depth) {
+            if (t < count) {
+                ct->sums[t] = sub[cur][t];
+                sum_of[cur][t] = t;
+            }
+            nsums = count;
+            __syncthreads();
+        }
     }
     if (bad) {
-        atomicOr(status, 2);
-        na = 0;
+        if (t == 0) atomicOr(status, 2);
+        count = nsums = 0;
     }
-    for (int e = 0; e < na; ++e) fr[e] = a[e];
-    *count = na;
+    if (t < count) {
+        ct->units[t] = sub[cur][t];
+        const int s = sum_of[cur][t];
+        if (t == 0 || sum_of[cur][t - 1] != s) ct->first[s] = t;
+    }
+    if (t == 0) {
+        ct->first[nsums] = count;
+        if (bad) ct->first[0] = ct->first[1] = 0;
+        ct->nsums = nsums;
+        ct->nunits = count;
+    }
 }
 
-// Sorted point p: the frontier entries' partial sums in entry order, then the
-// per-point factors.
-template <typename PT, typename VT>
-__global__ void walk_combine_kernel(int n, const PT *__restrict__ spts, const uint32_t *__restrict__ idx,
-                                    const VT *__restrict__ part, const int *__restrict__ count, double2 *frep,
-                                    double *zi)
+// Sorted point p: the partial sums of the cut's subtrees in subtree order,
+// then the per-point factors.  Four lanes per point, one per quantity, in
+// blocks of one warp: the float64 adds and conversions (4 x 64 of each at the
+// deepest cut) go to a pipe of two lanes a cycle per SM, so a small problem
+// wants them on as many SMs as possible (N = 2000: 38 us with 8 blocks of 256
+// points' threads, 6 us with 250 warps).
+constexpr int kCombineBlock = 32;
+
+template <typename PT, typename T>
+__global__ void __launch_bounds__(kCombineBlock) walk_combine_kernel(int n, const PT *__restrict__ spts,
+                                                                     const uint32_t *__restrict__ idx,
+                                                                     const T *__restrict__ part,
+                                                                     const int *__restrict__ count, double2 *frep,
+                                                                     double *zi)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int nf = *count;
-    double rx = 0, ry = 0, rs = 0, z = 0;
-    for (int e = 0; e < nf; ++e) {
-        const VT v = part[(size_t)e * n + p];
-        rx += (double)v.x;
-        ry += (double)v.y;
-        rs += (double)v.z;
-        z += (double)v.w;
-    }
+    const int p = (blockIdx.x * kCombineBlock + threadIdx.x) >> 2, q = threadIdx.x & 3;
+    const int k = min(p, n - 1), nf = *count;
+    const T *__restrict__ v = part + 4 * (size_t)k + q;
+    double a = 0;
+#pragma unroll 8
+    for (int e = 0; e < nf; ++e) a += (double)v[4 * (size_t)e * n];
+    const double rx = __shfl_sync(0xffffffffu, a, 0, 4), ry = __shfl_sync(0xffffffffu, a, 1, 4);
+    const double rs = __shfl_sync(0xffffffffu, a, 2, 4), z = __shfl_sync(0xffffffffu, a, 3, 4);
+    if (p >= n || q > 0) return;
     double x, y, il;
     point_xy_il(spts[p], x, y, il);
     const double rsd = il * rs;
@@ -600,7 +1077,6 @@ __global__ void walk_combine_kernel(int n, const PT *__restrict__ spts, const ui
     frep[i] = make_double2(4.0 * il * (rx + rsd * x), 4.0 * il * (ry + rsd * y));
     zi[i] = z;
 }
-
 
 // Exact repulsion: one thread per point i, tiles of kExactBlock points j
 // staged in shared memory, every pair j != i of the same segment.  A small
@@ -746,10 +1222,51 @@ __global__ void exact_combine_kernel(const PT *__restrict__ pts, ExactArgs A)
 
 int walk_split_capacity(int64_t n)
 {
-    // frontier entries x points of the partial-sum buffer (0: no split)
+    // subtrees x points of the partial-sum buffer (0: no split)
     if (n <= 0 || n > kSplitMaxN) return 0;
     return (int)std::min<int64_t>(kMaxFrontier, kSplitEntries / n);
 }
+
+// Listed or direct: up to kListMaxN points (1,024 chunks) the direct walk's
+// few chains of visits leave the GPU idle (N = 20,011: 412 us direct against
+// 142 us to list and 133 us to sum); above, its chunks are enough and listing
+// costs more instructions than it saves time (N = 70,000: 363 us direct,
+// 173 + 172 us listed; list_units 0).  The tree is divided into enough units
+// for about kListWarps (chunk, unit) warps (N = 20,011, list kernel: 20,000 /
+// 40,000 / 100,000 warps 183 / 142 / 205 us).
+#ifndef LW
+#define LW 40000
+#endif
+#ifndef LMAX
+#define LMAX 128
+#endif
+constexpr int64_t kListWarps = LW;
+constexpr int64_t kListMaxN = 1 << 15;
+
+static int list_target(int64_t n)
+{
+    const int64_t chunks = std::max<int64_t>((n + 31) / 32, 1);
+    return (int)std::max<int64_t>(2, std::min<int64_t>(kListWarps / chunks, LMAX));
+}
+
+// First pages per chunk: the cap of the cut into units (a cut by point counts
+// overshoots its target; a cut at depth D has up to 4^D subtrees).
+int list_units(int64_t n)
+{
+    if (n > kListMaxN) return 0;
+    return std::min(kMaxUnits, std::max(4 * list_target(n), walk_split_capacity(n)));
+}
+
+// Further pages per pool: 512 pages a chunk (16,384 interactions; theta = 0.5
+// lists about 1,000 to 4,000 a chunk), 134 MB at kListMaxN points.
+static int list_per_pool(int64_t n) { return (int)((n + 31) / 32 * 512 / kListPools + 1); }
+
+int64_t list_pages(int64_t n)
+{
+    return n > kListMaxN ? 0 : (n + 31) / 32 * list_units(n) + (int64_t)list_per_pool(n) * kListPools;
+}
+size_t list_page_bytes() { return sizeof(uint2) * kPage; }
+int64_t list_flags(int64_t n) { return kListPools + (n + 31) / 32; }
 
 // Cut depth for n points: the shallowest that gives about 2048 warps, within
 // the buffer; `want` >= 0 overrides (clamped), -1 chooses.  (A deeper cut for
@@ -776,28 +1293,35 @@ void launch_walk(hts_ctx *c)
     const bool cnt = c->counters_on != 0;  // counters accumulate while enabled
     const bool seg = c->nseg > 1;
     const SegView sv{c->keys, c->seg_off, c->pre};
-    const int depth = seg ? 0 : walk_split_depth(n, c->walk_split, c->cfg.precision == HTS_FP64);
-    SplitView sp{nullptr, nullptr, nullptr};
+    const bool fp64 = c->cfg.precision == HTS_FP64;
+    const int depth = seg ? 0 : walk_split_depth(n, c->walk_split, fp64);
+    const bool list = !fp64 && !seg && !cnt && list_units(n) > 0;
+    SplitView sp{nullptr, nullptr};
+    const AnnulusView an{c->minmax, seg ? c->keys : nullptr, c->cfg.split_rule, n - 1};
     dim3 grid((unsigned)((warps * 32 + wb - 1) / wb), 1);
-    if (depth > 0) {
-        Frontier *fr = reinterpret_cast<Frontier *>(c->split_frontier);
-        int *fcount = reinterpret_cast<int *>(fr + kMaxFrontier);
-        if (c->cfg.precision == HTS_FP32_MIXED)
-            frontier_kernel<<<1, 32, 0, c->stream>>>(NodesF{c->nodes32}, c->n_nodes, n, depth, fr, fcount, c->status);
+    if (list || depth > 0) {
+        CutTables *ct = reinterpret_cast<CutTables *>(c->split_frontier);
+        const int grain = list ? std::max(32, n / list_target(n)) : INT_MAX, cap = list ? list_units(n) : kMaxFrontier;
+        if (!fp64)
+            cut_kernel<<<1, kMaxUnits, 0, c->stream>>>(NodesF{c->nodes32}, c->n_nodes, n, depth, grain, cap, ct,
+                                                       c->status);
         else
-            frontier_kernel<<<1, 32, 0, c->stream>>>(NodesD{c->nodes64}, c->n_nodes, n, depth, fr, fcount, c->status);
+            cut_kernel<<<1, kMaxUnits, 0, c->stream>>>(NodesD{c->nodes64}, c->n_nodes, n, depth, grain, cap, ct,
+                                                       c->status);
         c->launches += 1;
-        sp = SplitView{fr, fcount, c->split_part};
+        sp = SplitView{ct, c->split_part};
         grid.y = 1u << (2 * depth);
     }
     c->launches += 1;
     // blocks in order of their cost in the previous walk, when the grid is
     // more than one wave (resident threads per SM: 2048)
-    const bool balance = depth == 0 && (int64_t)grid.x > (int64_t)c->sm_count * (2048 / wb);
+    const bool balance = !list && depth == 0 && (int64_t)grid.x > (int64_t)c->sm_count * (2048 / wb);
     const BlockOrder bo{balance ? c->walk_order : nullptr, balance ? c->walk_cost : nullptr};
 #define HTS_WALK(P, NODES, SPTS, GF, CT, SG, SPL)                                                    \
-    walk_##P##_kernel<GF, CT, SG, SPL><<<grid, wb, 0, c->stream>>>(n, NODES, c->n_nodes, SPTS, c->idx,   \
-                                                                   c->frep, c->zi, c->counters, sv, sp, bo)
+    walk_##P##_kernel<GF, CT, SG, SPL><<<grid, wb, 0, c->stream>>>(n, NODES, c->n_nodes, SPTS, c->cnt, c->idx, \
+                                                                   c->frep, c->zi, c->counters, sv, sp HTS_X##P, bo)
+#define HTS_Xf32 , an
+#define HTS_Xf64
 #define HTS_WALK_GF(P, NODES, SPTS, GF)                                                                   \
     if (depth > 0) {                                                                                       \
         if (cnt) HTS_WALK(P, NODES, SPTS, GF, true, false, true); else HTS_WALK(P, NODES, SPTS, GF, false, false, true); \
@@ -806,41 +1330,54 @@ void launch_walk(hts_ctx *c)
     } else {                                                                                               \
         if (seg) HTS_WALK(P, NODES, SPTS, GF, false, true, false); else HTS_WALK(P, NODES, SPTS, GF, false, false, false); \
     }
+#define HTS_SUM(GF, SPL)                                                                                          \
+    sum_f32_kernel<GF, SPL><<<dim3((unsigned)warps, grid.y), 32 * kSumWarps, 0, c->stream>>>(n, c->nodes32, c->n_nodes, c->spts32, c->cnt, c->idx, c->frep, \
+                                                        c->zi, sp, lv, an)
 #define HTS_WALK_ALL(P, NODES, SPTS)                                \
     if (c->cfg.grad_form == HTS_EXACT_KL) {                          \
         HTS_WALK_GF(P, NODES, SPTS, 0)                               \
     } else {                                                         \
         HTS_WALK_GF(P, NODES, SPTS, 1)                               \
     }
-    if (c->cfg.precision == HTS_FP32_MIXED) {
-        const NodesF nf{c->nodes32};
-        HTS_WALK_ALL(f32, nf, c->spts32)
+    if (list) {
+        const ListView lv{c->list_entries, c->list_head, c->list_flags, c->list_flags + kListPools, list_units(n),
+                          warps, list_per_pool(n)};
+        cudaMemsetAsync(c->list_flags, 0, sizeof(int) * (size_t)list_flags(n), c->stream);
+        list_f32_kernel<<<dim3((unsigned)((warps * 32 + kListBlock - 1) / kListBlock), (unsigned)lv.units), kListBlock,
+                          0, c->stream>>>(n, c->nodes32, c->spts32, c->cnt, sp.cut, lv);
+        c->launches += 1;
+        if (c->cfg.grad_form == HTS_EXACT_KL) {
+            if (depth > 0) HTS_SUM(0, true); else HTS_SUM(0, false);
+        } else {
+            if (depth > 0) HTS_SUM(1, true); else HTS_SUM(1, false);
+        }
+    } else if (!fp64) {
+        HTS_WALK_ALL(f32, c->nodes32, c->spts32)
     } else {
         HTS_WALK_ALL(f64, c->nodes64, c->spts64)
     }
-#undef HTS_WALK_ALL
-#undef HTS_WALK_GF
-#undef HTS_WALK
     if (balance) {
         walk_order_kernel<<<1, 1024, 0, c->stream>>>(c->walk_cost, (int)grid.x, c->walk_order);
         c->launches += 1;
     }
+#undef HTS_WALK_ALL
+#undef HTS_SUM
+#undef HTS_WALK
+#undef HTS_WALK_GF
     if (depth > 0) {
-        const int cb = (n + 255) / 256;
-        const int *fcount = reinterpret_cast<const int *>(reinterpret_cast<Frontier *>(c->split_frontier) +
-                                                          kMaxFrontier);
-        if (c->cfg.precision == HTS_FP32_MIXED)
-            walk_combine_kernel<PointF, float4><<<cb, 256, 0, c->stream>>>(
-                n, c->spts32, c->idx, reinterpret_cast<const float4 *>(c->split_part), fcount, c->frep, c->zi);
+        const unsigned cb = (unsigned)(((int64_t)n * 4 + kCombineBlock - 1) / kCombineBlock);
+        const int *nsums = &reinterpret_cast<const CutTables *>(c->split_frontier)->nsums;
+        if (!fp64)
+            walk_combine_kernel<PointF, float><<<cb, kCombineBlock, 0, c->stream>>>(
+                n, c->spts32, c->idx, reinterpret_cast<const float *>(c->split_part), nsums, c->frep, c->zi);
         else
-            walk_combine_kernel<PointD, double4_32a><<<cb, 256, 0, c->stream>>>(
-                n, c->spts64, c->idx, reinterpret_cast<const double4_32a *>(c->split_part), fcount, c->frep,
-                c->zi);
+            walk_combine_kernel<PointD, double><<<cb, kCombineBlock, 0, c->stream>>>(
+                n, c->spts64, c->idx, reinterpret_cast<const double *>(c->split_part), nsums, c->frep, c->zi);
         c->launches += 1;
     }
 }
 
-size_t walk_split_frontier_bytes() { return sizeof(Frontier) * kMaxFrontier + 64; }
+size_t walk_split_frontier_bytes() { return sizeof(CutTables); }
 
 int exact_split(int64_t n)
 {

@@ -403,7 +403,8 @@ struct EmitArgs {
     const double2 *y;
     const PointF *spts32;
     const PointD *spts64;
-    const int *left, *parent, *leaf_parent, *lo_arr, *hi_arr, *pref, *quad, *cnt, *pre;
+    const int *left, *parent, *leaf_parent, *lo_arr, *hi_arr, *pref, *quad, *pre;
+    int *cnt;
     const unsigned *mask;
     const FX3 *prefix;  // n + 1 exclusive prefix sums of the Einstein terms (fixed point)
     const unsigned long long *gmax;  // largest gamma (bits): the fixed-point exponent
@@ -419,9 +420,9 @@ __global__ void emit_kernel(EmitArgs A)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = A.n;
-    if (k == 0 && A.nodes32) {  // four empty slots after the last node: the float32 walk's overrun
+    if (k == 0 && A.nodes32) {  // empty slots after the last node: the float32 walk's overrun
         const int m = min(A.pre[n], A.capacity);
-        for (int e = 0; e < kWalkOverrun; ++e) A.nodes32[m + e] = NodeF{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0};
+        for (int e = 0; e < kWalkOverrun; ++e) A.nodes32[m + e] = NodeF{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, m + e + 1};
     }
     if (k < n - 1 && A.quad[k]) {
         int lo = A.lo_arr[k], hi = A.hi_arr[k];
@@ -491,8 +492,8 @@ __global__ void emit_kernel(EmitArgs A)
             split_f32(cx, nd.xh, nd.xl);
             split_f32(cy, nd.yh, nd.yl);
             split_f32(beta, b32, unused);  // (float)beta
-            nd.il = __frcp_rn(b32);
-            nd.thr = bucket ? __int_as_float(lo) : thr32;
+            nd.il = bucket ? __int_as_float(lo) : __frcp_rn(b32);
+            nd.thr = bucket ? -1.0f : thr32;
             nd.count = bucket ? -count : count;
             nd.skip = skip;
             A.nodes32[pos] = nd;
@@ -526,8 +527,9 @@ __global__ void emit_kernel(EmitArgs A)
     }
     if (k < n) {
         bool leaf = n == 1 || quad_level(A.pref[A.leaf_parent[k]]) < kLevels;
-        if (!leaf) return;
         int pos = A.pre[k] + A.cnt[k] - 1;
+        A.cnt[k] = leaf ? pos : -1;  // from here on: the position of the point's own leaf
+        if (!leaf) return;
         if (pos < 0 || pos >= A.capacity) {
             atomicOr(A.status, 2);
             return;
@@ -540,7 +542,7 @@ __global__ void emit_kernel(EmitArgs A)
             nd.xl = q.xl;
             nd.yl = q.yl;
             nd.il = q.il;
-            nd.thr = __int_as_float(k);
+            nd.thr = -1.0f;
             nd.count = 1;
             nd.skip = pos + 1;
             A.nodes32[pos] = nd;
