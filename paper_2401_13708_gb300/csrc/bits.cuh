@@ -7,6 +7,7 @@
 // arithmetic.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -18,6 +19,17 @@ __host__ __device__ __forceinline__ unsigned long long bits_of(double x)
     return (unsigned long long)__double_as_longlong(x);
 #else
     unsigned long long b;
+    memcpy(&b, &x, sizeof b);
+    return b;
+#endif
+}
+
+__host__ __device__ __forceinline__ unsigned bits_of(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    unsigned b;
     memcpy(&b, &x, sizeof b);
     return b;
 #endif
