@@ -116,12 +116,12 @@ int ensure_points(hts_ctx *c, int64_t n)
         AL(c->pts32, N);
         AL(c->apts32, N);
         AL(c->spts32, N);
-        AL(c->nodes32, 2 * N + kWalkOverrun);
     } else {
         AL(c->pts64, N);
         AL(c->spts64, N);
         AL(c->nodes64, 2 * N);
     }
+    AL(c->nodes32, 2 * N + kWalkOverrun);  // (in float64 mode they decide the criterion)
     // a node slot never written by a tree build reads as an empty bucket
     // (count 0), which the walk steps over (its skip is its index + 1)
     if (c->nodes32) {
@@ -174,8 +174,8 @@ int ensure_points(hts_ctx *c, int64_t n)
         c->split_part = part;
         c->split_frontier = fr;
     }
-    if (c->cfg.precision == HTS_FP32_MIXED) {
-        const size_t pages = (size_t)list_pages((int64_t)N);
+    {
+        const size_t pages = (size_t)list_pages((int64_t)N, c->cfg.precision == HTS_FP64);
         AL(c->list_entries, pages * (list_page_bytes() / sizeof(uint2)));
         AL(c->list_head, pages);
         AL(c->list_flags, (size_t)list_flags((int64_t)N));

@@ -239,7 +239,7 @@ int walk_split_capacity(int64_t n);
 int walk_split_depth(int64_t n, int want, bool fp64);
 size_t walk_split_frontier_bytes();
 // interaction lists: pages for n points, bytes of a page, counters and flags
-int64_t list_pages(int64_t n);
+int64_t list_pages(int64_t n, bool fp64);
 size_t list_page_bytes();
 int64_t list_flags(int64_t n);
 // attract.cu

@@ -24,6 +24,7 @@
 // written to the point's original index.
 #include <limits.h>
 
+
 #include <algorithm>
 
 #include "hts_internal.cuh"
@@ -137,16 +138,10 @@ struct SplitView {
     void *part;                       // [sum][n] partial sums (float4 / double4); nullptr: one sum
 };
 
-struct NodesF {  // float32 nodes: cell test, points and skip index
+struct NodesF {  // cell test, points and skip index
     const NodeF *nodes;
     __device__ bool cell(int k) const { return nodes[k].count >= 2.0f; }
     __device__ int points(int k) const { return (int)nodes[k].count; }
-    __device__ int skip(int k) const { return nodes[k].skip; }
-};
-struct NodesD {  // float64 nodes
-    const NodeD *nodes;
-    __device__ bool cell(int k) const { return nodes[k].count >= 2; }
-    __device__ int points(int k) const { return nodes[k].count; }
     __device__ int skip(int k) const { return nodes[k].skip; }
 };
 
@@ -215,6 +210,16 @@ struct BatchF {
 };
 constexpr int kBatchFull = 28;  // evaluated above this (a trip of the walk adds up to four)
 
+// Notes an interaction that some lane takes.
+__device__ __forceinline__ void batch_add(BatchF &B, int lane, int node, unsigned m)
+{
+    if (lane == B.count) {
+        B.node = node;
+        B.mask = m;
+    }
+    B.count += m != 0u ? 1 : 0;
+}
+
 // Node data of a batch, one array per field, so that the data of consecutive
 // interactions are register pairs of one (broadcast) shared-memory load.
 struct __align__(16) TileF {
@@ -240,11 +245,7 @@ __device__ __forceinline__ int visit_f32(int node, int end, int lane, LaneF &L, 
     const unsigned m = __ballot_sync(0xffffffffu, acc);
     const bool down = __any_sync(0xffffffffu, open && !acc);
     if (acc) L.resume = c.skip;
-    if (lane == B.count) {
-        B.node = node;
-        B.mask = m;
-    }
-    B.count += m != 0u ? 1 : 0;
+    batch_add(B, lane, node, m);
     // next > node always: every node slot's skip exceeds its index
     return down ? node + 1 : c.skip;
 }
@@ -342,12 +343,7 @@ __device__ __forceinline__ bool visit_ancestors_f32(const Cut &F, bool live, int
         float s;
         delta_f32(L, make_float2(a.xh, a.yh), make_float2(a.xl, a.yl), s);
         const bool acc = live && s * L.twoil * a.il > a.thr;
-        const unsigned m = __ballot_sync(0xffffffffu, acc && own);
-        if (lane == B.count) {
-            B.node = at;
-            B.mask = m;
-        }
-        B.count += m != 0u ? 1 : 0;
+        batch_add(B, lane, at, __ballot_sync(0xffffffffu, acc && own));
         live = live && !acc;
     }
     return live;
@@ -543,6 +539,38 @@ __global__ void __launch_bounds__(kWalkBlock) walk_f32_kernel(int n, const NodeF
     record_cost(bo, b, t0);
 }
 
+// The page a (chunk, unit) warp writes its batches to.
+struct ListPage {
+    int page;
+    __device__ ListPage(const ListView &lv, int chunk, int unit) : page(chunk * lv.units + unit) {}
+    __device__ __forceinline__ void write(const ListView &lv, int lane, const BatchF &B) const
+    {
+        if (lane < B.count) lv.entries[(size_t)page * kPage + lane] = make_uint2((unsigned)B.node, B.mask);
+    }
+    // The batch fills the page: writes it and takes another (false: none left).
+    __device__ __forceinline__ bool next(const ListView &lv, int chunk, int lane, BatchF &B)
+    {
+        write(lv, lane, B);
+        const int pool = chunk & (kListPools - 1);
+        int to = 0;
+        if (lane == 0) {
+            to = atomicAdd(&lv.taken[pool], 1);
+            to = to < lv.per_pool ? lv.chunks * lv.units + pool * lv.per_pool + to : -1;
+            lv.head[page] = make_int2(B.count, to);
+            if (to < 0) lv.direct[chunk] = 1;
+        }
+        to = __shfl_sync(0xffffffffu, to, 0);
+        page = to;
+        B.count = 0;
+        return to >= 0;
+    }
+    __device__ __forceinline__ void last(const ListView &lv, int lane, const BatchF &B) const
+    {
+        write(lv, lane, B);
+        if (lane == 0) lv.head[page] = make_int2(B.count, -1);
+    }
+};
+
 // Lists the interactions of a chunk (grid.x: chunks, a warp each; the warps of
 // a block take consecutive chunks, so their walks share node data in L1) with
 // one unit of the tree (grid.y).
@@ -565,28 +593,13 @@ __global__ void __launch_bounds__(kListBlock, 6) list_f32_kernel(int n, const No
     const int end = F.end;
     L.resume = live ? node : INT_MAX;
     if (!__any_sync(0xffffffffu, live)) node = end;
-    int page = chunk * lv.units + (int)blockIdx.y;
-    const int pool = chunk & (kListPools - 1);
+    ListPage page(lv, chunk, (int)blockIdx.y);
     while (node < end) {  // (a page holds what a trip can add to kBatchFull)
 #pragma unroll
         for (int k = 0; k < kPage - kBatchFull; ++k) node = visit_f32(node, end, lane, L, B, nodes);
-        if (B.count > kBatchFull) {  // the page is full: write it, take another
-            if (lane < B.count) lv.entries[(size_t)page * kPage + lane] = make_uint2((unsigned)B.node, B.mask);
-            int next = 0;
-            if (lane == 0) {
-                next = atomicAdd(&lv.taken[pool], 1);
-                next = next < lv.per_pool ? lv.chunks * lv.units + pool * lv.per_pool + next : -1;
-                lv.head[page] = make_int2(B.count, next);
-                if (next < 0) lv.direct[chunk] = 1;
-            }
-            next = __shfl_sync(0xffffffffu, next, 0);
-            if (next < 0) return;
-            page = next;
-            B.count = 0;
-        }
+        if (B.count > kBatchFull && !page.next(lv, chunk, lane, B)) return;
     }
-    if (lane < B.count) lv.entries[(size_t)page * kPage + lane] = make_uint2((unsigned)B.node, B.mask);
-    if (lane == 0) lv.head[page] = make_int2(B.count, -1);
+    page.last(lv, lane, B);
 }
 
 // A block evaluates the listed interactions of a chunk (grid.x; grid.y: the
@@ -756,115 +769,278 @@ __global__ void __launch_bounds__(32 * kSumWarps, 6) sum_f32_kernel(int n, const
     store_lane(L, sum, n, idx, frep, zi, SPLIT ? sp.part : nullptr);
 }
 
-template <int GF, bool COUNT, bool SEG, bool SPLIT>
-__device__ __forceinline__ void walk_f64_chunk(int warp, int n, const NodeD *__restrict__ nodes,
-                                                const int *__restrict__ n_nodes,
-                                                const PointD *__restrict__ spts,
-                                                const uint32_t *__restrict__ idx, double2 *frep, double *zi,
-                                                unsigned long long *counters, const SegView sv,
-                                                const SplitView sp, int fi)
+// ---- float64 walk ---------------------------------------------------------
+// The float64 pipe (two lanes a cycle per SM) bounds it, so float64 is spent
+// on the pair terms alone, on lanes that need them:
+//   - the criterion is decided in float32 from the float32 nodes, whose
+//     positions are hi/lo pairs, wherever the float32 delta is further from
+//     the threshold than its error; otherwise (about one test in 10^5) in
+//     float64, so every decision is the float64 one;
+//   - accepted interactions go to a ring of four groups of 32, and every lane
+//     takes its own ones in order: a lane that takes few in one group goes on
+//     to the next while the others catch up (a lane takes about 70% of its
+//     warp's interactions).
+// Walk at N = 70,000, theta = 0.5: 15.1 ms visit by visit, 10.1 ms with whole
+// batches of 128, 8.2 ms with the ring; 21.6 ms before the pair terms of
+// f64math.cuh.
+constexpr int kWalkBlockD = 128;
+constexpr float kSureF32 = 3.8146973e-6f;   // 2^-18
+constexpr float kNearF32 = 8.8817842e-16f;  // 2^-50
+
+struct __align__(16) TileD {
+    double2 xy[128];
+    double2 ic[128];   // conformal factor; points (negative: a bucket)
+    int node[128];
+    unsigned mask[128];
+};
+
+struct LaneD {
+    double x, y, twoil;
+    double rx, ry, rs, z;
+    float2 qh, ql;  // the position as hi / lo float pairs
+    float twoilf;
+    int p, own, resume;
+};
+
+__device__ __forceinline__ void load_lane(LaneD &L, int chunk, int lane, int n, const PointD *__restrict__ spts,
+                                          const int *__restrict__ leaf)
 {
-    const int lane = threadIdx.x & 31;
-    const int p = warp * 32 + lane;
-    const bool valid = p < n;
-    const PointD q = spts[valid ? p : n - 1];
-    const double twoil = 2.0 * q.il;
-    double rx = 0, ry = 0, rs = 0, z = 0;
-    const int m = min(*n_nodes, 2 * n);
-    int root = 0, end = m;
-    if (SEG) segment_range(sv, valid ? p : n - 1, m, root, end);
-    unsigned long long c_acc = 0, c_pair = 0, c_visit = 0;
-    bool live = valid;
-    if (SPLIT) {  // as in the float32 walk
-        const Cut &F = sp.cut->sums[fi];
-        for (int k = 0; k < F.nanc; ++k) {
-            const NodeD a = nodes[F.anc[k]];
-            double dx = q.x - a.x, dy = q.y - a.y;
-            double s = fma(dx, dx, dy * dy);
-            double delta = s * twoil * a.il;
-            if (live && delta > a.thr) {
-                if ((F.own >> k) & 1) {
-                    PairD t = pair_terms_f64<GF>(delta);
-                    double mult = (double)a.count;
-                    double kk = mult * t.rep * a.il;
-                    rx = fma(kk, dx, rx);
-                    ry = fma(kk, dy, ry);
-                    rs = fma(kk, s, rs);
-                    z = fma(mult, t.w, z);
-                    if (COUNT) ++c_acc;
-                }
-                live = false;
+    L.p = chunk * 32 + lane;
+    const int k = min(L.p, n - 1);
+    const PointD q = spts[k];
+    L.x = q.x;
+    L.y = q.y;
+    L.twoil = 2.0 * q.il;
+    split_f32(q.x, L.qh.x, L.ql.x);
+    split_f32(q.y, L.qh.y, L.ql.y);
+    L.twoilf = (float)L.twoil;
+    L.own = leaf[k];
+    L.rx = L.ry = L.rs = L.z = 0.0;
+}
+
+template <int GF>
+__device__ __forceinline__ void add_pair_f64(LaneD &L, double x, double y, double il, double mult)
+{
+    const double dx = L.x - x, dy = L.y - y;
+    const double s = fma(dx, dx, dy * dy);
+    const PairD t = pair_terms_f64<GF>(s * L.twoil * il);
+    const double k = mult * t.rep * il;
+    L.rx = fma(k, dx, L.rx);
+    L.ry = fma(k, dy, L.ry);
+    L.rs = fma(k, s, L.rs);
+    L.z = fma(mult, t.w, L.z);
+}
+
+// A depth-29 bucket: each of its points (not the lane's own).
+template <int GF>
+__device__ __forceinline__ void add_bucket_f64(LaneD &L, int node, const NodeD *__restrict__ nodes64,
+                                               const PointD *__restrict__ spts, int n, unsigned &pairs)
+{
+    const NodeD c = nodes64[node];
+    const int lo = c.pos, cnt = -c.count;
+    if (lo < 0 || cnt <= 0 || lo + cnt > n) return;
+    for (int k = 0; k < cnt; ++k) {
+        if (lo + k == L.p) continue;
+        const PointD o = spts[lo + k];
+        add_pair_f64<GF>(L, o.x, o.y, o.il, 1.0);
+        ++pairs;
+    }
+}
+
+// A lane's criterion at a node (r_cell / d < theta  <=>  delta > thr); `ask`:
+// the lane is open there.  The float32 delta is off by less than 2^-20 of
+// itself where |Delta| > 2^-25: the compensated difference by 3 x 2^-24 of
+// itself and 2^-47, il, thr and the products by a few 2^-24 more; 2^-18 is
+// allowed.  Leaves and buckets have threshold -1.
+__device__ __forceinline__ bool accepts_f64(const LaneD &L, bool ask, const NodeF &c, int node,
+                                            const NodeD *__restrict__ nodes64)
+{
+    const float2 d = delta2(L.qh, L.ql, make_float2(c.xh, c.yh), make_float2(c.xl, c.yl));
+    const float s = fmaf(d.x, d.x, d.y * d.y);
+    const float delta = s * L.twoilf * c.il, margin = c.thr * kSureF32;
+    bool acc = delta > c.thr;
+    const bool unsure = ask && c.count >= 2.0f && (fabsf(delta - c.thr) <= margin || s < kNearF32) && c.thr < 3e38f;
+    if (__any_sync(0xffffffffu, unsure)) {
+        if (unsure) {
+            const NodeD e = nodes64[node];
+            const double dx = L.x - e.x, dy = L.y - e.y;
+            acc = fma(dx, dx, dy * dy) * L.twoil * e.il > e.thr;
+        }
+        __syncwarp();
+    }
+    return ask && acc;
+}
+
+// One visit (as visit_f32); `m`: the lanes that take the node's interaction.
+__device__ __forceinline__ int visit_f64(int node, int end, LaneD &L, unsigned &m, const NodeF *__restrict__ nodes,
+                                         const NodeD *__restrict__ nodes64)
+{
+    const NodeF c = load_node(nodes, node);
+    const bool open = node >= L.resume && node < end;
+    const bool acc = accepts_f64(L, open && node != L.own, c, node, nodes64);
+    m = __ballot_sync(0xffffffffu, acc);
+    const bool down = __any_sync(0xffffffffu, open && !acc);
+    if (acc) L.resume = c.skip;
+    return down ? node + 1 : c.skip;
+}
+
+// The ring: group i of those held (0: the oldest) is at (head + i) mod 4 of the
+// warp's tile; bit e of b_i: the lane has interaction e of group i to add.
+struct RingD {
+    unsigned b0, b1, b2, b3;
+    int head, held;
+};
+
+// The nodes and masks of `count` interactions of the next group are in the
+// tile: fetches their data.
+__device__ __forceinline__ void ring_push(RingD &R, int count, int lane, TileD &T, const NodeD *__restrict__ nodes64)
+{
+    __syncwarp();
+    const int e = ((R.head + R.held) & 3) * 32 + lane;
+    const bool have = lane < count;
+    if (have) {
+        const NodeD c = nodes64[T.node[e]];
+        T.xy[e] = make_double2(c.x, c.y);
+        T.ic[e] = make_double2(c.il, (double)c.count);
+    }
+    const unsigned b = transpose_bits(have ? T.mask[e] : 0u, lane);
+    R.b0 = R.held == 0 ? b : R.b0;
+    R.b1 = R.held == 1 ? b : R.b1;
+    R.b2 = R.held == 2 ? b : R.b2;
+    R.b3 = R.held == 3 ? b : R.b3;
+    ++R.held;
+    __syncwarp();
+}
+
+// Adds interactions until every lane is done with the oldest group, and frees it.
+template <int GF>
+__device__ __forceinline__ void ring_drain(RingD &R, LaneD &L, TileD &T, const NodeD *__restrict__ nodes64,
+                                           const PointD *__restrict__ spts, int n, unsigned &pairs)
+{
+    while (__any_sync(0xffffffffu, R.b0 != 0u)) {
+        int e = -1;  // the lane's next interaction
+        if (R.b0) {
+            e = __ffs((int)R.b0) - 1;
+            R.b0 &= R.b0 - 1u;
+        } else if (R.b1) {
+            e = __ffs((int)R.b1) + 31;
+            R.b1 &= R.b1 - 1u;
+        } else if (R.b2) {
+            e = __ffs((int)R.b2) + 63;
+            R.b2 &= R.b2 - 1u;
+        } else if (R.b3) {
+            e = __ffs((int)R.b3) + 95;
+            R.b3 &= R.b3 - 1u;
+        }
+        __syncwarp();
+        if (e >= 0) {
+            e = (e + 32 * R.head) & 127;
+            const double2 xy = T.xy[e], ic = T.ic[e];
+            if ((long long)bits_of(ic.y) > 0) {
+                add_pair_f64<GF>(L, xy.x, xy.y, ic.x, ic.y);
+            } else {
+                add_bucket_f64<GF>(L, T.node[e], nodes64, spts, n, pairs);
             }
+        }
+        __syncwarp();
+    }
+    R.b0 = R.b1;
+    R.b1 = R.b2;
+    R.b2 = R.b3;
+    R.b3 = 0u;
+    R.head = (R.head + 1) & 3;
+    --R.held;
+}
+
+__device__ __forceinline__ void store_lane(const LaneD &L, int sum, int n, const uint32_t *__restrict__ idx,
+                                           double2 *frep, double *zi, void *part)
+{
+    if (L.p >= n) return;
+    if (part) {
+        reinterpret_cast<double4_32a *>(part)[(size_t)sum * n + L.p] = make_double4_32a(L.rx, L.ry, L.rs, L.z);
+        return;
+    }
+    const uint32_t i = idx[L.p];
+    const double il = 0.5 * L.twoil, rsd = il * L.rs;
+    frep[i] = make_double2(4.0 * il * (L.rx + rsd * L.x), 4.0 * il * (L.ry + rsd * L.y));
+    zi[i] = L.z;
+}
+
+// One warp walks for a chunk (sum `sum` of the cut when there are partial sums).
+template <int GF, bool COUNT, bool SEG, bool SPLIT>
+__device__ __forceinline__ void walk_f64_chunk(LaneD &L, int n, int lane, const NodeF *__restrict__ nodes,
+                                                const NodeD *__restrict__ nodes64, const int *__restrict__ n_nodes,
+                                                const PointD *__restrict__ spts, unsigned long long *counters,
+                                                const SegView sv, const CutTables *cut, int sum, TileD &T)
+{
+    unsigned long long c_visit = 0, c_acc = 0, c_pair = 0;
+    const bool valid = L.p < n;
+    const int m = min(*n_nodes, 2 * n);
+    int root = 0, end = m, count = 0;
+    if (SEG) segment_range(sv, valid ? L.p : n - 1, m, root, end);
+    bool live = valid;
+    RingD R{0u, 0u, 0u, 0u, 0, 0};
+    if (SPLIT) {  // ancestors first, then the subtree [node, end)
+        const Cut &F = cut->sums[sum];
+        const int na = F.nanc, owned = F.own;
+        for (int k = 0; k < na; ++k) {
+            const int at = F.anc[k];
+            const bool own = (owned >> k) & 1;
+            const bool acc = accepts_f64(L, live, load_node(nodes, at), at, nodes64);
+            const unsigned am = __ballot_sync(0xffffffffu, acc && own);
+            if (am != 0u) {
+                if (lane == 0) {
+                    T.node[count] = at;
+                    T.mask[count] = am;
+                }
+                ++count;
+            }
+            if (COUNT) c_acc += (acc && own) ? 1 : 0;
+            live = live && !acc;
         }
         root = F.node;
         end = F.end;
     }
-    int resume = live ? root : INT_MAX;
-    int node = SEG ? __shfl_sync(0xffffffffu, root, 0) : root;
-    const int stop = SEG ? __reduce_max_sync(0xffffffffu, valid ? end : 0) : end;
-    while (node < stop) {
-        const NodeD c = nodes[node];
-        const bool active = node >= resume && (!SEG || node < end);
-        int next = node + 1;
-        if (c.count >= 2) {
-            double dx = q.x - c.x, dy = q.y - c.y;
-            double s = fma(dx, dx, dy * dy);
-            double delta = s * twoil * c.il;
-            bool acc = active && delta > c.thr;
-            if (acc) {
-                PairD t = pair_terms_f64<GF>(delta);
-                double mult = (double)c.count;
-                double k = mult * t.rep * c.il;
-                rx = fma(k, dx, rx);
-                ry = fma(k, dy, ry);
-                rs = fma(k, s, rs);
-                z = fma(mult, t.w, z);
-                resume = c.skip;
-                if (COUNT) ++c_acc;
-            }
-            if (!__any_sync(0xffffffffu, active && !acc)) next = c.skip;
-        } else if (c.count == 1) {
-            if (active && c.pos != p) {
-                double dx = q.x - c.x, dy = q.y - c.y;
-                double s = fma(dx, dx, dy * dy);
-                PairD t = pair_terms_f64<GF>(s * twoil * c.il);
-                double k = t.rep * c.il;
-                rx = fma(k, dx, rx);
-                ry = fma(k, dy, ry);
-                rs = fma(k, s, rs);
-                z += t.w;
-                if (COUNT) ++c_pair;
-            }
-        } else {
-            const int lo = c.pos, cnt = -c.count;
-            if (active && lo >= 0 && cnt > 0 && lo + cnt <= n) {
-                for (int k2 = 0; k2 < cnt; ++k2) {
-                    if (lo + k2 == p) continue;
-                    PointD o = spts[lo + k2];
-                    double dx = q.x - o.x, dy = q.y - o.y;
-                    double s = fma(dx, dx, dy * dy);
-                    PairD t = pair_terms_f64<GF>(s * twoil * o.il);
-                    double k = t.rep * o.il;
-                    rx = fma(k, dx, rx);
-                    ry = fma(k, dy, ry);
-                    rs = fma(k, s, rs);
-                    z += t.w;
-                    if (COUNT) ++c_pair;
+    L.resume = live ? root : INT_MAX;
+    int node = SEG ? __shfl_sync(0xffffffffu, root, 0) : root;  // lane 0 holds the first segment
+    int stop = SEG ? __reduce_max_sync(0xffffffffu, valid ? end : 0) : end;
+    if (!__any_sync(0xffffffffu, live)) stop = node;
+    unsigned pairs = 0;
+    while (true) {
+        while (R.held < 4 && node < stop) {  // fill the next group
+            const int base = ((R.head + R.held) & 3) * 32;
+            while (count < 32 && node < stop) {
+                unsigned am;
+                const int at = node;
+                if (COUNT && lane == 0) ++c_visit;
+                node = visit_f64(node, end, L, am, nodes, nodes64);
+                if (am != 0u) {
+                    if (lane == 0) {
+                        T.node[base + count] = at;
+                        T.mask[base + count] = am;
+                    }
+                    ++count;
+                    if (COUNT && ((am >> lane) & 1u)) {
+                        const float ct = nodes[at].count;
+                        c_acc += ct >= 2.0f ? 1 : 0;
+                        c_pair += ct == 1.0f ? 1 : 0;
+                    }
                 }
             }
+            if (count == 32) {
+                ring_push(R, 32, lane, T, nodes64);
+                count = 0;
+            }
         }
-        if (COUNT && lane == 0) ++c_visit;
-        node = next;  // as in the float32 walk
-    }
-    if (SPLIT && valid) {
-        reinterpret_cast<double4_32a *>(sp.part)[(size_t)fi * n + p] = make_double4_32a(rx, ry, rs, z);
-    } else if (valid) {
-        const uint32_t i = idx[p];
-        double rsd = q.il * rs;
-        frep[i] = make_double2(4.0 * q.il * (rx + rsd * q.x), 4.0 * q.il * (ry + rsd * q.y));
-        zi[i] = z;
+        if (count > 0 && R.held < 4) {  // the last interactions
+            ring_push(R, count, lane, T, nodes64);
+            count = 0;
+        }
+        if (R.held == 0) break;
+        ring_drain<GF>(R, L, T, nodes64, spts, n, pairs);
     }
     if (COUNT) {
+        c_pair += pairs;
         for (int o = 16; o > 0; o >>= 1) {
             c_acc += __shfl_xor_sync(0xffffffffu, c_acc, o);
             c_pair += __shfl_xor_sync(0xffffffffu, c_pair, o);
@@ -873,29 +1049,220 @@ __device__ __forceinline__ void walk_f64_chunk(int warp, int n, const NodeD *__r
             atomicAdd(&counters[0], c_acc);
             atomicAdd(&counters[1], c_pair);
             atomicAdd(&counters[2], c_visit);
-            atomicAdd(&counters[3], (unsigned long long)min(32, n - warp * 32));
+            atomicAdd(&counters[3], (unsigned long long)min(32, n - L.p));
         }
     }
 }
 
-// As walk_f32_kernel, in float64.
+// Direct walk: one warp per chunk of 32 sorted points (grid.x) and sum (grid.y).
 template <int GF, bool COUNT, bool SEG, bool SPLIT>
-__global__ void __launch_bounds__(kWalkBlock) walk_f64_kernel(int n, const NodeD *__restrict__ nodes,
-                                                              const int *__restrict__ n_nodes,
-                                                              const PointD *__restrict__ spts,
-                                                              const int *__restrict__ leaf,
-                                                              const uint32_t *__restrict__ idx, double2 *frep,
-                                                              double *zi, unsigned long long *counters,
-                                                              const SegView sv, const SplitView sp,
-                                                              const BlockOrder bo)
+__global__ void __launch_bounds__(kWalkBlockD) walk_f64_kernel(int n, const NodeF *__restrict__ nodes,
+                                                               const NodeD *__restrict__ nodes64,
+                                                               const int *__restrict__ n_nodes,
+                                                               const PointD *__restrict__ spts,
+                                                               const int *__restrict__ leaf,
+                                                               const uint32_t *__restrict__ idx, double2 *frep,
+                                                               double *zi, unsigned long long *counters,
+                                                               const SegView sv, const SplitView sp,
+                                                               const BlockOrder bo)
 {
+    __shared__ TileD tile[kWalkBlockD / 32];
     const int b = logical_block(bo);
-    const int warp = (b * blockDim.x + threadIdx.x) >> 5;
-    if (warp * 32 >= n) return;
+    const int chunk = (b * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (chunk * 32 >= n) return;
     if (SPLIT && (int)blockIdx.y >= sp.cut->nsums) return;
     const long long t0 = clock64();
-    walk_f64_chunk<GF, COUNT, SEG, SPLIT>(warp, n, nodes, n_nodes, spts, idx, frep, zi, counters, sv, sp, blockIdx.y);
+    LaneD L;
+    load_lane(L, chunk, lane, n, spts, leaf);
+    walk_f64_chunk<GF, COUNT, SEG, SPLIT>(L, n, lane, nodes, nodes64, n_nodes, spts, counters, sv, sp.cut, blockIdx.y,
+                                          tile[threadIdx.x >> 5]);
+    store_lane(L, blockIdx.y, n, idx, frep, zi, SPLIT ? sp.part : nullptr);
     record_cost(bo, b, t0);
+}
+
+// Small problems: lists the interactions of a chunk with one unit of the tree,
+// as list_f32_kernel.
+__global__ void __launch_bounds__(kListBlock, 6) list_f64_kernel(int n, const NodeF *__restrict__ nodes,
+                                                                 const NodeD *__restrict__ nodes64,
+                                                                 const PointD *__restrict__ spts,
+                                                                 const int *__restrict__ leaf,
+                                                                 const CutTables *__restrict__ cut, const ListView lv)
+{
+    const int chunk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (chunk >= lv.chunks || (int)blockIdx.y >= cut->nunits) return;
+    LaneD L;
+    load_lane(L, chunk, lane, n, spts, leaf);
+    BatchF B;
+    B.node = 0;
+    B.mask = 0u;
+    B.count = 0;
+    const Cut &F = cut->units[blockIdx.y];
+    bool live = L.p < n;
+    const int na = F.nanc, owned = F.own;
+    for (int k = 0; k < na; ++k) {
+        const int at = F.anc[k];
+        const bool own = (owned >> k) & 1;
+        const bool acc = accepts_f64(L, live, load_node(nodes, at), at, nodes64);
+        batch_add(B, lane, at, __ballot_sync(0xffffffffu, acc && own));
+        live = live && !acc;
+    }
+    int node = F.node;
+    const int end = F.end;
+    L.resume = live ? node : INT_MAX;
+    if (!__any_sync(0xffffffffu, live)) node = end;
+    ListPage page(lv, chunk, (int)blockIdx.y);
+    while (node < end) {
+#pragma unroll 1
+        for (int k = 0; k < kPage - kBatchFull; ++k) {
+            unsigned m;
+            const int at = node;
+            node = visit_f64(node, end, L, m, nodes, nodes64);
+            batch_add(B, lane, at, m);
+        }
+        if (B.count > kBatchFull && !page.next(lv, chunk, lane, B)) return;
+    }
+    page.last(lv, lane, B);
+}
+
+// Blocks evaluate the listed interactions of a chunk (grid.x), a window of up
+// to kWindow at a time: in every window a point's interactions are divided
+// evenly among the lanes that hold the point, one in each of the warps of the
+// chunk's blocks (grid.y), so that the float64 pipe sees full warps whatever
+// the lists look like (it is busy 87% of the kernel at N = 70,000; one pair
+// term is 39 float64 operations).  The lanes' sums are added in warp order (of several
+// blocks: by walk_combine_kernel), so the result is reproducible.
+constexpr int kSumBlockD = 192;
+constexpr int kWindow = 320;  // (256 - 768 interactions and 4 - 8 warps: within 5% of each other)
+
+struct WindowD {
+    double2 xy[kWindow];
+    double2 ic[kWindow];                 // conformal factor; points (negative: a bucket)
+    int node[kWindow];
+    unsigned take[kWindow / 32][32];     // [batch][lane]: the interactions of the batch that the lane's point takes
+    double4_32a sums[kSumBlockD / 32][32];
+};
+
+template <int GF>
+__device__ __forceinline__ void sum_window_f64(LaneD &L, int batches, int share, int shares, int lane, const WindowD &W,
+                                               const NodeD *__restrict__ nodes64, const PointD *__restrict__ spts, int n)
+{
+    int total = 0;
+    for (int b = 0; b < batches; ++b) total += __popc(W.take[b][lane]);
+    int at = total * share / shares, left = total * (share + 1) / shares - at;  // the lane's share of the point's
+    int b = -1;
+    unsigned bits = 0u;
+    while (__any_sync(0xffffffffu, left > 0)) {
+        if (left > 0) {
+            while (true) {  // to the next interaction
+                const int here = __popc(bits);
+                if (at < here) break;
+                at -= here;
+                bits = W.take[++b][lane];
+            }
+            for (; at > 0; --at) bits &= bits - 1u;
+            const int e = 32 * b + __ffs((int)bits) - 1;
+            bits &= bits - 1u;
+            --left;
+            const double2 xy = W.xy[e], ic = W.ic[e];
+            if ((long long)bits_of(ic.y) > 0) {
+                add_pair_f64<GF>(L, xy.x, xy.y, ic.x, ic.y);
+            } else {
+                unsigned pairs = 0;
+                add_bucket_f64<GF>(L, W.node[e], nodes64, spts, n, pairs);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <int GF>
+__global__ void __launch_bounds__(kSumBlockD) sum_f64_kernel(int n, const NodeF *__restrict__ nodes,
+                                                             const NodeD *__restrict__ nodes64,
+                                                             const int *__restrict__ n_nodes,
+                                                             const PointD *__restrict__ spts,
+                                                             const int *__restrict__ leaf,
+                                                             const uint32_t *__restrict__ idx, double2 *frep,
+                                                             double *zi, const SplitView sp, const ListView lv)
+{
+    constexpr int kWarps = kSumBlockD / 32, kBatches = kWindow / 32;
+    __shared__ union { WindowD window; TileD tile; } S;
+    WindowD &W = S.window;
+    const int chunk = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int shares = kWarps * (int)gridDim.y, share = (int)blockIdx.y * kWarps + w;
+    LaneD L;
+    load_lane(L, chunk, lane, n, spts, leaf);
+    if (lv.direct[chunk]) {  // (the same for the whole block)
+        if (share > 0) return;
+        walk_f64_chunk<GF, false, false, false>(L, n, lane, nodes, nodes64, n_nodes, spts, nullptr, SegView{}, nullptr,
+                                                0, S.tile);
+        store_lane(L, 0, n, idx, frep, zi, gridDim.y > 1 ? sp.part : nullptr);
+        return;
+    }
+    // batches of up to 32 interactions from consecutive pages, dealt to the
+    // warps to fetch; every warp follows the same pages
+    int slot = 0, fill = 0;
+    const int units = sp.cut->nunits;
+    unsigned mask = 0u;
+    auto done = [&]() {
+        if (slot % kWarps == w) {
+            __syncwarp();
+            const int e = 32 * slot + lane;
+            if (lane < fill) {
+                const NodeD c = nodes64[W.node[e]];
+                W.xy[e] = make_double2(c.x, c.y);
+                W.ic[e] = make_double2(c.il, (double)c.count);
+            }
+            W.take[slot][lane] = transpose_bits(lane < fill ? mask : 0u, lane);
+        }
+        ++slot;
+        fill = 0;
+    };
+    auto flush = [&]() {
+        __syncthreads();
+        sum_window_f64<GF>(L, slot, share, shares, lane, W, nodes64, spts, n);
+        __syncthreads();
+        slot = 0;
+    };
+    for (int ub = 0; ub < units; ub += 32) {
+        const int2 h = ub + lane < units ? lv.head[chunk * lv.units + ub + lane] : make_int2(0, -1);
+        unsigned todo = __ballot_sync(0xffffffffu, h.x > 0);
+        while (todo) {
+            const int j = __ffs((int)todo) - 1;
+            todo &= todo - 1;
+            int page = chunk * lv.units + ub + j;
+            int count = __shfl_sync(0xffffffffu, h.x, j), next = __shfl_sync(0xffffffffu, h.y, j);
+            while (true) {
+                if (fill + count > 32) {
+                    done();
+                    if (slot == kBatches) flush();
+                }
+                if (slot % kWarps == w && lane >= fill && lane < fill + count) {
+                    const uint2 e = lv.entries[(size_t)page * kPage + lane - fill];
+                    W.node[32 * slot + lane] = (int)e.x;
+                    mask = e.y;
+                }
+                fill += count;
+                if (next < 0) break;
+                page = next;
+                const int2 g = lv.head[page];
+                count = g.x;
+                next = g.y;
+            }
+        }
+    }
+    if (fill > 0) done();
+    if (slot > 0) flush();
+    W.sums[w][lane] = make_double4_32a(L.rx, L.ry, L.rs, L.z);
+    __syncthreads();
+    if (w > 0) return;
+    for (int k = 1; k < kWarps; ++k) {
+        const double4_32a v = W.sums[k][lane];
+        L.rx += v.x;
+        L.ry += v.y;
+        L.rs += v.z;
+        L.z += v.w;
+    }
+    store_lane(L, blockIdx.y, n, idx, frep, zi, gridDim.y > 1 ? sp.part : nullptr);
 }
 
 // The next launch order from the recorded costs: a counting sort on 256
@@ -941,8 +1308,7 @@ __global__ void __launch_bounds__(1024) walk_order_kernel(unsigned *cost, int nb
 // cell with more than 4 children or a skip that does not advance is a broken
 // tree: status bit 2, no subtrees (the walk then does no work and the error is
 // reported).
-template <typename NV>
-__global__ void __launch_bounds__(kMaxUnits) cut_kernel(const NV nodes, const int *__restrict__ n_nodes, int n,
+__global__ void __launch_bounds__(kMaxUnits) cut_kernel(const NodesF nodes, const int *__restrict__ n_nodes, int n,
                                                         int depth, int grain, int cap, CutTables *ct, int *status)
 {
     __shared__ Cut sub[2][kMaxUnits];
@@ -1046,8 +1412,8 @@ __global__ void __launch_bounds__(kMaxUnits) cut_kernel(const NV nodes, const in
     }
 }
 
-// Sorted point p: the partial sums of the cut's subtrees in subtree order,
-// then the per-point factors.  Four lanes per point, one per quantity, in
+// The partial sums of a point in order (the cut's subtrees, or the chunks of
+// the exact kernel), then the per-point factors.  Four lanes per point, one per quantity, in
 // blocks of one warp: the float64 adds and conversions (4 x 64 of each at the
 // deepest cut) go to a pipe of two lanes a cycle per SM, so a small problem
 // wants them on as many SMs as possible (N = 2000: 38 us with 8 blocks of 256
@@ -1058,11 +1424,11 @@ template <typename PT, typename T>
 __global__ void __launch_bounds__(kCombineBlock) walk_combine_kernel(int n, const PT *__restrict__ spts,
                                                                      const uint32_t *__restrict__ idx,
                                                                      const T *__restrict__ part,
-                                                                     const int *__restrict__ count, double2 *frep,
-                                                                     double *zi)
+                                                                     const int *__restrict__ count, int fixed,
+                                                                     double2 *frep, double *zi)
 {
     const int p = (blockIdx.x * kCombineBlock + threadIdx.x) >> 2, q = threadIdx.x & 3;
-    const int k = min(p, n - 1), nf = *count;
+    const int k = min(p, n - 1), nf = count ? *count : fixed;
     const T *__restrict__ v = part + 4 * (size_t)k + q;
     double a = 0;
 #pragma unroll 8
@@ -1073,7 +1439,7 @@ __global__ void __launch_bounds__(kCombineBlock) walk_combine_kernel(int n, cons
     double x, y, il;
     point_xy_il(spts[p], x, y, il);
     const double rsd = il * rs;
-    const uint32_t i = idx[p];
+    const uint32_t i = idx ? idx[p] : (uint32_t)p;  // sorted positions, or points
     frep[i] = make_double2(4.0 * il * (rx + rsd * x), 4.0 * il * (ry + rsd * y));
     zi[i] = z;
 }
@@ -1083,7 +1449,7 @@ __global__ void __launch_bounds__(kCombineBlock) walk_combine_kernel(int n, cons
 // problem has too few i-blocks to fill the GPU, so the j range of each
 // i-block is cut into `split` chunks (grid.y): with split == 1 the block
 // writes the finished force and Z_i, otherwise raw sums per chunk go to
-// `part` and exact_combine_kernel adds them in chunk order (deterministic).
+// `part` and walk_combine_kernel adds them in chunk order (deterministic).
 struct ExactArgs {
     int n, split;
     double2 *frep;
@@ -1196,28 +1562,6 @@ __global__ void __launch_bounds__(kExactBlock) exact_f64_kernel(const PointD *__
     A.zi[i] = z;
 }
 
-// Sums of the chunks of each point in chunk order, then the per-point factors.
-template <typename PT>
-__global__ void exact_combine_kernel(const PT *__restrict__ pts, ExactArgs A)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= A.n) return;
-    double rx = 0, ry = 0, rs = 0, z = 0;
-    for (int c = 0; c < A.split; ++c) {
-        const double4_32a v = A.part[(size_t)c * A.n + i];
-        rx += v.x;
-        ry += v.y;
-        rs += v.z;
-        z += v.w;
-    }
-    const PT q = pts[i];
-    double x, y, il;
-    point_xy_il(q, x, y, il);
-    const double rsd = il * rs;
-    A.frep[i] = make_double2(4.0 * il * (rx + rsd * x), 4.0 * il * (ry + rsd * y));
-    A.zi[i] = z;
-}
-
 }  // namespace
 
 int walk_split_capacity(int64_t n)
@@ -1233,7 +1577,9 @@ int walk_split_capacity(int64_t n)
 // costs more instructions than it saves time (N = 70,000: 363 us direct,
 // 173 + 172 us listed; list_units 0).  The tree is divided into enough units
 // for about kListWarps (chunk, unit) warps (N = 20,011, list kernel: 20,000 /
-// 40,000 / 100,000 warps 183 / 142 / 205 us).
+// 40,000 / 100,000 warps 183 / 142 / 205 us).  In float64 the pair terms are
+// most of the walk and the listed ones fill the float64 pipe better (N =
+// 70,000: 8.2 ms direct, 0.5 + 7.3 ms listed), so the limit is the lists' size.
 #ifndef LW
 #define LW 40000
 #endif
@@ -1241,7 +1587,7 @@ int walk_split_capacity(int64_t n)
 #define LMAX 128
 #endif
 constexpr int64_t kListWarps = LW;
-constexpr int64_t kListMaxN = 1 << 15;
+constexpr int64_t kListMaxN = 1 << 15, kListMaxN64 = 1 << 18;
 
 static int list_target(int64_t n)
 {
@@ -1251,19 +1597,21 @@ static int list_target(int64_t n)
 
 // First pages per chunk: the cap of the cut into units (a cut by point counts
 // overshoots its target; a cut at depth D has up to 4^D subtrees).
-int list_units(int64_t n)
+int list_units(int64_t n, bool fp64)
 {
-    if (n > kListMaxN) return 0;
+    if (n > (fp64 ? kListMaxN64 : kListMaxN)) return 0;
     return std::min(kMaxUnits, std::max(4 * list_target(n), walk_split_capacity(n)));
 }
 
 // Further pages per pool: 512 pages a chunk (16,384 interactions; theta = 0.5
-// lists about 1,000 to 4,000 a chunk), 134 MB at kListMaxN points.
-static int list_per_pool(int64_t n) { return (int)((n + 31) / 32 * 512 / kListPools + 1); }
+// lists about 1,000 to 4,000 a chunk), 134 MB at kListMaxN points; above, 256
+// a chunk, 537 MB at kListMaxN64.
+static int list_per_pool(int64_t n) { return (int)((n + 31) / 32 * (n > kListMaxN ? 256 : 512) / kListPools + 1); }
 
-int64_t list_pages(int64_t n)
+int64_t list_pages(int64_t n, bool fp64)
 {
-    return n > kListMaxN ? 0 : (n + 31) / 32 * list_units(n) + (int64_t)list_per_pool(n) * kListPools;
+    const int u = list_units(n, fp64);
+    return u ? (n + 31) / 32 * u + (int64_t)list_per_pool(n) * kListPools : 0;
 }
 size_t list_page_bytes() { return sizeof(uint2) * kPage; }
 int64_t list_flags(int64_t n) { return kListPools + (n + 31) / 32; }
@@ -1285,6 +1633,15 @@ int walk_split_depth(int64_t n, int want, bool fp64)
     return d;
 }
 
+// Blocks per chunk that sum a listed float64 walk: four blocks per SM while
+// there are fewer chunks than SMs (N = 2,000, two / four / six per SM: 124 /
+// 108 / 132 us).
+static int f64_sum_blocks(const hts_ctx *c)
+{
+    const int64_t chunks = std::max<int64_t>((c->n + 31) / 32, 1);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(4 * c->sm_count / chunks, std::min(16, walk_split_capacity(c->n))));
+}
+
 void launch_walk(hts_ctx *c)
 {
     const int n = (int)c->n;
@@ -1295,19 +1652,19 @@ void launch_walk(hts_ctx *c)
     const SegView sv{c->keys, c->seg_off, c->pre};
     const bool fp64 = c->cfg.precision == HTS_FP64;
     const int depth = seg ? 0 : walk_split_depth(n, c->walk_split, fp64);
-    const bool list = !fp64 && !seg && !cnt && list_units(n) > 0;
+    // (float64: a depth that was asked for is the cut of the direct walk)
+    const bool list = !seg && (!fp64 || c->walk_split < 0) && !cnt && list_units(n, fp64) > 0;
+    const int blocks64 = fp64 && list ? f64_sum_blocks(c) : 1;
+    const bool split = fp64 && list ? blocks64 > 1 : depth > 0;
     SplitView sp{nullptr, nullptr};
     const AnnulusView an{c->minmax, seg ? c->keys : nullptr, c->cfg.split_rule, n - 1};
-    dim3 grid((unsigned)((warps * 32 + wb - 1) / wb), 1);
-    if (list || depth > 0) {
-        CutTables *ct = reinterpret_cast<CutTables *>(c->split_frontier);
-        const int grain = list ? std::max(32, n / list_target(n)) : INT_MAX, cap = list ? list_units(n) : kMaxFrontier;
-        if (!fp64)
-            cut_kernel<<<1, kMaxUnits, 0, c->stream>>>(NodesF{c->nodes32}, c->n_nodes, n, depth, grain, cap, ct,
-                                                       c->status);
-        else
-            cut_kernel<<<1, kMaxUnits, 0, c->stream>>>(NodesD{c->nodes64}, c->n_nodes, n, depth, grain, cap, ct,
-                                                       c->status);
+    const int wbd = std::min(wb, kWalkBlockD);
+    const int block = fp64 ? wbd : wb;
+    dim3 grid((unsigned)((warps * 32 + block - 1) / block), 1);
+    CutTables *ct = reinterpret_cast<CutTables *>(c->split_frontier);
+    if (list || split) {
+        const int grain = list ? std::max(32, n / list_target(n)) : INT_MAX, cap = list ? list_units(n, fp64) : kMaxFrontier;
+        cut_kernel<<<1, kMaxUnits, 0, c->stream>>>(NodesF{c->nodes32}, c->n_nodes, n, depth, grain, cap, ct, c->status);
         c->launches += 1;
         sp = SplitView{ct, c->split_part};
         grid.y = 1u << (2 * depth);
@@ -1315,64 +1672,74 @@ void launch_walk(hts_ctx *c)
     c->launches += 1;
     // blocks in order of their cost in the previous walk, when the grid is
     // more than one wave (resident threads per SM: 2048)
-    const bool balance = !list && depth == 0 && (int64_t)grid.x > (int64_t)c->sm_count * (2048 / wb);
+    const bool balance = !list && !split && (int64_t)grid.x > (int64_t)c->sm_count * (2048 / block);
     const BlockOrder bo{balance ? c->walk_order : nullptr, balance ? c->walk_cost : nullptr};
-#define HTS_WALK(P, NODES, SPTS, GF, CT, SG, SPL)                                                    \
-    walk_##P##_kernel<GF, CT, SG, SPL><<<grid, wb, 0, c->stream>>>(n, NODES, c->n_nodes, SPTS, c->cnt, c->idx, \
-                                                                   c->frep, c->zi, c->counters, sv, sp HTS_X##P, bo)
-#define HTS_Xf32 , an
-#define HTS_Xf64
-#define HTS_WALK_GF(P, NODES, SPTS, GF)                                                                   \
-    if (depth > 0) {                                                                                       \
-        if (cnt) HTS_WALK(P, NODES, SPTS, GF, true, false, true); else HTS_WALK(P, NODES, SPTS, GF, false, false, true); \
-    } else if (cnt) {                                                                                      \
-        if (seg) HTS_WALK(P, NODES, SPTS, GF, true, true, false); else HTS_WALK(P, NODES, SPTS, GF, true, false, false); \
-    } else {                                                                                               \
-        if (seg) HTS_WALK(P, NODES, SPTS, GF, false, true, false); else HTS_WALK(P, NODES, SPTS, GF, false, false, false); \
+#define HTS_WALK32(GF, CT, SG, SPL)                                                                                  \
+    walk_f32_kernel<GF, CT, SG, SPL><<<grid, block, 0, c->stream>>>(n, c->nodes32, c->n_nodes, c->spts32, c->cnt, \
+                                                                    c->idx, c->frep, c->zi, c->counters, sv, sp, an, bo)
+#define HTS_WALK64(GF, CT, SG, SPL)                                                                             \
+    walk_f64_kernel<GF, CT, SG, SPL><<<grid, block, 0, c->stream>>>(n, c->nodes32, c->nodes64, c->n_nodes,   \
+                                                                    c->spts64, c->cnt, c->idx, c->frep, c->zi, \
+                                                                    c->counters, sv, sp, bo)
+#define HTS_SUM(GF, CT, SG, SPL)                                                                                     \
+    sum_f32_kernel<GF, SPL><<<dim3((unsigned)warps, grid.y), 32 * kSumWarps, 0, c->stream>>>(                        \
+        n, c->nodes32, c->n_nodes, c->spts32, c->cnt, c->idx, c->frep, c->zi, sp, lv, an)
+#define HTS_WALK_GF(K, GF)                                                                       \
+    if (split) {                                                                                 \
+        if (cnt) K(GF, true, false, true); else K(GF, false, false, true);                       \
+    } else if (cnt) {                                                                            \
+        if (seg) K(GF, true, true, false); else K(GF, true, false, false);                       \
+    } else {                                                                                     \
+        if (seg) K(GF, false, true, false); else K(GF, false, false, false);                     \
     }
-#define HTS_SUM(GF, SPL)                                                                                          \
-    sum_f32_kernel<GF, SPL><<<dim3((unsigned)warps, grid.y), 32 * kSumWarps, 0, c->stream>>>(n, c->nodes32, c->n_nodes, c->spts32, c->cnt, c->idx, c->frep, \
-                                                        c->zi, sp, lv, an)
-#define HTS_WALK_ALL(P, NODES, SPTS)                                \
-    if (c->cfg.grad_form == HTS_EXACT_KL) {                          \
-        HTS_WALK_GF(P, NODES, SPTS, 0)                               \
-    } else {                                                         \
-        HTS_WALK_GF(P, NODES, SPTS, 1)                               \
+#define HTS_WALK(K)                                \
+    if (c->cfg.grad_form == HTS_EXACT_KL) {        \
+        HTS_WALK_GF(K, 0)                          \
+    } else {                                       \
+        HTS_WALK_GF(K, 1)                          \
     }
     if (list) {
-        const ListView lv{c->list_entries, c->list_head, c->list_flags, c->list_flags + kListPools, list_units(n),
+        const ListView lv{c->list_entries, c->list_head, c->list_flags, c->list_flags + kListPools, list_units(n, fp64),
                           warps, list_per_pool(n)};
         cudaMemsetAsync(c->list_flags, 0, sizeof(int) * (size_t)list_flags(n), c->stream);
-        list_f32_kernel<<<dim3((unsigned)((warps * 32 + kListBlock - 1) / kListBlock), (unsigned)lv.units), kListBlock,
-                          0, c->stream>>>(n, c->nodes32, c->spts32, c->cnt, sp.cut, lv);
+        const dim3 lgrid((unsigned)((warps * 32 + kListBlock - 1) / kListBlock), (unsigned)lv.units);
         c->launches += 1;
-        if (c->cfg.grad_form == HTS_EXACT_KL) {
-            if (depth > 0) HTS_SUM(0, true); else HTS_SUM(0, false);
+        if (fp64) {
+            list_f64_kernel<<<lgrid, kListBlock, 0, c->stream>>>(n, c->nodes32, c->nodes64, c->spts64, c->cnt, sp.cut, lv);
+            const dim3 sgrid((unsigned)warps, (unsigned)blocks64);
+            if (c->cfg.grad_form == HTS_EXACT_KL)
+                sum_f64_kernel<0><<<sgrid, kSumBlockD, 0, c->stream>>>(n, c->nodes32, c->nodes64, c->n_nodes, c->spts64,
+                                                                        c->cnt, c->idx, c->frep, c->zi, sp, lv);
+            else
+                sum_f64_kernel<1><<<sgrid, kSumBlockD, 0, c->stream>>>(n, c->nodes32, c->nodes64, c->n_nodes, c->spts64,
+                                                                        c->cnt, c->idx, c->frep, c->zi, sp, lv);
         } else {
-            if (depth > 0) HTS_SUM(1, true); else HTS_SUM(1, false);
+            list_f32_kernel<<<lgrid, kListBlock, 0, c->stream>>>(n, c->nodes32, c->spts32, c->cnt, sp.cut, lv);
+            HTS_WALK(HTS_SUM)
         }
-    } else if (!fp64) {
-        HTS_WALK_ALL(f32, c->nodes32, c->spts32)
+    } else if (fp64) {
+        HTS_WALK(HTS_WALK64)
     } else {
-        HTS_WALK_ALL(f64, c->nodes64, c->spts64)
+        HTS_WALK(HTS_WALK32)
     }
     if (balance) {
         walk_order_kernel<<<1, 1024, 0, c->stream>>>(c->walk_cost, (int)grid.x, c->walk_order);
         c->launches += 1;
     }
-#undef HTS_WALK_ALL
-#undef HTS_SUM
 #undef HTS_WALK
 #undef HTS_WALK_GF
-    if (depth > 0) {
+#undef HTS_SUM
+#undef HTS_WALK64
+#undef HTS_WALK32
+    if (split) {
         const unsigned cb = (unsigned)(((int64_t)n * 4 + kCombineBlock - 1) / kCombineBlock);
-        const int *nsums = &reinterpret_cast<const CutTables *>(c->split_frontier)->nsums;
         if (!fp64)
             walk_combine_kernel<PointF, float><<<cb, kCombineBlock, 0, c->stream>>>(
-                n, c->spts32, c->idx, reinterpret_cast<const float *>(c->split_part), nsums, c->frep, c->zi);
+                n, c->spts32, c->idx, reinterpret_cast<const float *>(c->split_part), &ct->nsums, 0, c->frep, c->zi);
         else
             walk_combine_kernel<PointD, double><<<cb, kCombineBlock, 0, c->stream>>>(
-                n, c->spts64, c->idx, reinterpret_cast<const double *>(c->split_part), nsums, c->frep, c->zi);
+                n, c->spts64, c->idx, reinterpret_cast<const double *>(c->split_part), list ? nullptr : &ct->nsums, blocks64,
+                c->frep, c->zi);
         c->launches += 1;
     }
 }
@@ -1398,20 +1765,24 @@ void launch_exact(hts_ctx *c)
     A.seg_of = c->nseg > 1 ? c->seg_of : nullptr;
     A.seg_off = c->seg_off;
     const dim3 grid((unsigned)((A.n + kExactBlock - 1) / kExactBlock), (unsigned)A.split);
-    const int cb = (A.n + 255) / 256;
+    const unsigned cb = (unsigned)(((int64_t)A.n * 4 + kCombineBlock - 1) / kCombineBlock);
     c->launches += A.split > 1 ? 2 : 1;
     if (c->cfg.precision == HTS_FP32_MIXED) {
         if (c->cfg.grad_form == HTS_EXACT_KL)
             exact_f32_kernel<0><<<grid, kExactBlock, 0, c->stream>>>(c->pts32, A);
         else
             exact_f32_kernel<1><<<grid, kExactBlock, 0, c->stream>>>(c->pts32, A);
-        if (A.split > 1) exact_combine_kernel<PointF><<<cb, 256, 0, c->stream>>>(c->pts32, A);
+        if (A.split > 1)
+            walk_combine_kernel<PointF, double><<<cb, kCombineBlock, 0, c->stream>>>(A.n, c->pts32, nullptr, c->exact_part,
+                                                                                     nullptr, A.split, A.frep, A.zi);
     } else {
         if (c->cfg.grad_form == HTS_EXACT_KL)
             exact_f64_kernel<0><<<grid, kExactBlock, 0, c->stream>>>(c->pts64, A);
         else
             exact_f64_kernel<1><<<grid, kExactBlock, 0, c->stream>>>(c->pts64, A);
-        if (A.split > 1) exact_combine_kernel<PointD><<<cb, 256, 0, c->stream>>>(c->pts64, A);
+        if (A.split > 1)
+            walk_combine_kernel<PointD, double><<<cb, kCombineBlock, 0, c->stream>>>(A.n, c->pts64, nullptr, c->exact_part,
+                                                                                     nullptr, A.split, A.frep, A.zi);
     }
 }
 

@@ -492,7 +492,7 @@ __global__ void emit_kernel(EmitArgs A)
             split_f32(cx, nd.xh, nd.xl);
             split_f32(cy, nd.yh, nd.yl);
             split_f32(beta, b32, unused);  // (float)beta
-            nd.il = bucket ? __int_as_float(lo) : __frcp_rn(b32);
+            nd.il = bucket ? __int_as_float(lo) : A.nodes64 ? (float)il : __frcp_rn(b32);
             nd.thr = bucket ? -1.0f : thr32;
             nd.count = bucket ? -count : count;
             nd.skip = skip;
@@ -535,7 +535,15 @@ __global__ void emit_kernel(EmitArgs A)
             return;
         }
         if (A.nodes32) {
-            PointF q = A.spts32[k];
+            PointF q;
+            if (A.spts32) {
+                q = A.spts32[k];
+            } else {  // float64 mode: the float32 nodes decide its criterion
+                const PointD e = A.spts64[k];
+                split_f32(e.x, q.xh, q.xl);
+                split_f32(e.y, q.yh, q.yl);
+                q.il = (float)e.il;
+            }
             NodeF nd;
             nd.xh = q.xh;
             nd.yh = q.yh;
@@ -620,7 +628,7 @@ void launch_build_tree(hts_ctx *c, double theta, const TreeExport *ex)
     A.keys = c->keys;
     A.idx = c->idx;
     A.y = c->y;
-    A.spts32 = c->spts32;
+    A.spts32 = f32 ? c->spts32 : nullptr;
     A.spts64 = c->spts64;
     A.left = c->bn_left;
     A.parent = c->bn_parent;
@@ -635,7 +643,7 @@ void launch_build_tree(hts_ctx *c, double theta, const TreeExport *ex)
     A.prefix = prefix;
     A.mm = c->minmax;
     A.gmax = gmax;
-    A.nodes32 = f32 ? c->nodes32 : nullptr;
+    A.nodes32 = c->nodes32;
     A.nodes64 = f32 ? nullptr : c->nodes64;
     A.ex = ex ? *ex : TreeExport{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     A.capacity = 2 * n;

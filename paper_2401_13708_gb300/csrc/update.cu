@@ -80,6 +80,7 @@ struct UpdateArgs {
     const double *Z;
     double exag, lr, mom, eps;
     int metric_pow, use_gains, do_step;
+    int rounded;  // float64 mode: |y|^2 and long steps with every operation rounded on its own
     double2 *g_out;
     int *status;
     const double *xsq;  // CO-SNE |x_i|^2 (nullptr: off)
@@ -106,6 +107,25 @@ __device__ __forceinline__ double tanh_step(double x)
     return tanh(x);
 }
 
+// exp_p(v) with every operation rounded on its own (no fused multiply-adds, no
+// reciprocals), for steps of several units of hyperbolic length: there
+// 1 + 2 <p, u> + |p|^2 |u|^2 cancels to about (1 - |p|)^2, and one rounding
+// more or less in it moves a point at the rim by 1e-6.
+__device__ __noinline__ double2 long_step(double2 p, double2 v)
+{
+    const double n2 = __dadd_rn(__dmul_rn(p.x, p.x), __dmul_rn(p.y, p.y));
+    const double nv = __dsqrt_rn(__dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)));
+    const double lam = __ddiv_rn(2.0, __dsub_rn(1.0, n2));
+    const double t = tanh(__ddiv_rn(__dmul_rn(lam, nv), 2.0));
+    const double ux = __ddiv_rn(__dmul_rn(t, v.x), nv), uy = __ddiv_rn(__dmul_rn(t, v.y), nv);
+    const double pu = __dadd_rn(__dmul_rn(p.x, ux), __dmul_rn(p.y, uy));
+    const double nu = __dadd_rn(__dmul_rn(ux, ux), __dmul_rn(uy, uy));
+    const double ca = __dadd_rn(__dadd_rn(1.0, __dmul_rn(2.0, pu)), nu), cb = __dsub_rn(1.0, n2);
+    const double den = __dadd_rn(__dadd_rn(1.0, __dmul_rn(2.0, pu)), __dmul_rn(n2, nu));
+    return make_double2(__ddiv_rn(__dadd_rn(__dmul_rn(ca, p.x), __dmul_rn(cb, ux)), den),
+                        __ddiv_rn(__dadd_rn(__dmul_rn(ca, p.y), __dmul_rn(cb, uy)), den));
+}
+
 __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
 {
     __shared__ double s_invz;
@@ -130,7 +150,7 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     double gx = 4.0 * (A.exag * fa.x - fr.x * invZ);
     double gy = 4.0 * (A.exag * fa.y - fr.y * invZ);
     double2 p = A.y[i];
-    const double n2 = p.x * p.x + p.y * p.y;
+    const double n2 = A.rounded ? __dadd_rn(__dmul_rn(p.x, p.x), __dmul_rn(p.y, p.y)) : p.x * p.x + p.y * p.y;
     if (A.xsq) {  // CO-SNE: lambda1 g_KL - (4 lambda2 / n)(|x|^2 - |y|^2) y
         const double ns = A.seg_of ? (double)(A.seg_off[sg + 1] - A.seg_off[sg]) : (double)A.n;
         const double c = 4.0 * A.l2 / ns * (A.xsq[i] - n2);
@@ -167,14 +187,19 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
         // exp map: p (+) tanh(lambda |v| / 2) v / |v|, lambda |v| / 2 = |v| / a;
         // 1 / |v| from one reciprocal square root (no square root and division)
         const double rn = rsqrt(vv), nv = vv * rn;
-        const double f = tanh_step(nv / a) * rn;
-        const double ux = f * v.x, uy = f * v.y;
-        const double pu = p.x * ux + p.y * uy;
-        const double nu = ux * ux + uy * uy;
-        const double ca = 1.0 + 2.0 * pu + nu;
-        const double rden = 1.0 / (1.0 + 2.0 * pu + n2 * nu);
-        q.x = (ca * p.x + a * ux) * rden;
-        q.y = (ca * p.y + a * uy) * rden;
+        const double x = nv / a;
+        if (A.rounded && x > 2.0) {
+            q = long_step(p, v);
+        } else {
+            const double f = tanh_step(x) * rn;
+            const double ux = f * v.x, uy = f * v.y;
+            const double pu = p.x * ux + p.y * uy;
+            const double nu = ux * ux + uy * uy;
+            const double ca = 1.0 + 2.0 * pu + nu;
+            const double rden = 1.0 / (1.0 + 2.0 * pu + n2 * nu);
+            q.x = (ca * p.x + a * ux) * rden;
+            q.y = (ca * p.y + a * uy) * rden;
+        }
     }
     const double q2 = q.x * q.x + q.y * q.y;
     const double lim = 1.0 - A.eps / 2.0;
@@ -233,6 +258,7 @@ void launch_update(hts_ctx *c, double exag, double lr, double mom, double2 *g_ou
     A.metric_pow = c->cfg.metric_pow;
     A.use_gains = c->cfg.use_gains;
     A.do_step = do_step;
+    A.rounded = c->cfg.precision == HTS_FP64;
     A.g_out = g_out;
     A.status = c->status;
     A.xsq = c->xsq;

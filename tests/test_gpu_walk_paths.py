@@ -66,3 +66,26 @@ def test_lists_that_do_not_fit():
     interactions, more than its pool holds, and is walked directly."""
     g, z, g2, z2 = both(embedding(32768, 8.0, False), 0.01, 0)
     assert np.array_equal(g, g2) and z == z2
+
+
+# float64: the counting walk is the direct one (a ring per warp), the other
+# listed up to 262,144 points (several blocks per chunk below 304 chunks).
+# The same terms in another order: n 2^-53 of the terms' sum at most.
+@pytest.mark.parametrize("n", [1, 33, 64, 2049, 9729, 20001])
+@pytest.mark.parametrize("rho,theta", [(0.0, 0.5), (12.0, 0.2), (9.0, 1.0)])
+def test_float64_listed_and_direct(n, rho, theta):
+    y = embedding(n, rho, buckets=rho > 0)
+    with HyperbolicTSNE(precision="fp64") as t:
+        t.set_P(np.zeros(n + 1, np.int64), np.zeros(0, np.int32), np.zeros(0, np.float32))
+        t.set_Y(y)
+        g, z = t.grad(theta)
+        t.set_counters(True)
+        g2, z2 = t.grad(theta)
+        accepted = t.get_counters()[:2].copy()
+        t.set_counters(False)
+        t.set_counters(True)
+        t.set_walk_split(1)
+        t.grad(theta)
+        assert np.array_equal(t.get_counters()[:2], accepted)  # the same interactions, cut or not
+    assert abs(z - z2) <= 1e-12 * abs(z2)
+    assert np.linalg.norm(g - g2) <= 1e-12 * np.linalg.norm(g2) + 1e-300
