@@ -1,8 +1,10 @@
-// sort.cu -- LSD radix sort of (key, index) pairs and an exclusive int scan.
+// sort.cu -- sort of (key, index) pairs (by ranks, or an LSD radix sort) and an
+// exclusive int scan.
 //
 // The tree of Sec. 4.1 is a hierarchy over the keys, so sorting the points
-// by key puts every cell's points in one contiguous run.  Eight stable
-// passes of 8 bits each (58 key bits + 6 segment bits), one kernel per pass:
+// by key puts every cell's points in one contiguous run.  Up to kRankMax keys
+// they are sorted by ranks (sort_by_rank); above, eight stable passes of 8
+// bits each (58 key bits + 6 segment bits), one kernel per pass:
 //   digit_hist  once per sort: the global histograms of all eight digits
 //               (they do not depend on the order of the keys; shared-memory
 //               atomics per key and digit), then an exclusive scan of each
@@ -30,10 +32,21 @@
 namespace hts {
 namespace {
 
-constexpr int kSmallMax = 4096;    // up to this many keys, one block sorts (small_sort_kernel)
+// Sorted tiles and ranks (sort_by_rank) up to kRankMax keys, with larger tiles
+// for more keys: the tile sort grows with the tile, the rank search with their
+// number.  Measured (tile sort + ranks, us; radix sort's kernels, without the
+// gaps between its 11 launches):
+//   keys       512-key tiles  1024        2048         4096         radix
+//   2,000      4.1 + 4.3      7.1 + 4.1   13.7                      39.9
+//   8,192      4.2 + 8.4      7.2 + 5.6   14.0 + 5.0   31.7 + 4.1   42.1
+//   20,011     4.2 + 19.1     7.2 + 11.9  14.0 + 8.2   31.8 + 6.0   47.0
+//   40,000     4.3 + 37.2     7.2 + 21.1  14.0 + 13.7
+//   70,000                    7.3 + 49.5  14.1 + 29.0  31.8 + 18.1  55.9
+//   131,071                               14.1 + 48.2  31.7 + 26.9  60.8
+//   262,144                               14.1 + 177   31.8 + 95.5  76.4
+constexpr int64_t kRankMax = 150000, kRank512 = 8192, kRank1024 = 32768, kRank2048 = 90000;
 constexpr int kMinTile = 1024;     // one-sweep tiles hold 1024, 2048, 4096 or 8192 keys (tile_keys)
 constexpr int kSortThreads = 256;
-constexpr int kWarps = kSortThreads / 32;
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanBlock = kScanThreads * kScanItems;
@@ -326,87 +339,175 @@ int scan_exclusive(const int *in, int *out, int64_t len, int *tmp, cudaStream_t 
 
 namespace {
 
-// n <= kSmallMax: all eight passes in one block (no look-back: the block's own
-// histogram is the global one), ping-ponging through the two key buffers.
-// ROUNDS keys per lane: 256 * ROUNDS >= n (fewer rounds for fewer keys).
-template <int ROUNDS>
-__global__ void __launch_bounds__(kSortThreads) small_sort_kernel(uint64_t *ka, uint32_t *va, uint64_t *kb,
-                                                                  uint32_t *vb, int n)
+// ---- sort by ranks ------------------------------------------------------------
+// Up to kRankMax keys the eight dependent passes of the radix sort are latency
+// (11 launches), and comparing is cheaper.  A block
+// sorts a tile of kTile keys in shared memory: runs of 64 by counting the
+// smaller keys of the run, then runs of 512 and the tile by counting, for every
+// key, the smaller keys of each other run (binary searches).  One more kernel
+// finds every key's place among all tiles the same way, the first steps of
+// each search in a sample of every 32nd key.  Equal keys stay in index order:
+// runs and tiles hold consecutive indices, so an earlier one's equal keys come
+// before and a later one's after.  (A bitonic sort of a
+// 2,048-key tile: 22 us.)
+constexpr int kRun = 64, kRun2 = 512, kSample = 32;
+template <int kTile> constexpr int kTileThreads = kTile < 1024 ? kTile : 1024;
+
+// Keys of a sorted run (kLen, a power of two) that are below lim.
+template <int kLen>
+__device__ __forceinline__ int count_below(const uint64_t *run, uint64_t lim)
 {
-    constexpr int kRounds = ROUNDS;
-    __shared__ int wh[kWarps][256];
-    __shared__ int dsum[256];
-    __shared__ int wtot[kWarps];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const int base = w * 32 * ROUNDS;
-    for (int p = 0; p < kPasses; ++p) {
-        const uint64_t *kin = (p & 1) ? kb : ka;
-        const uint32_t *vin = (p & 1) ? vb : va;
-        uint64_t *kout = (p & 1) ? ka : kb;
-        uint32_t *vout = (p & 1) ? va : vb;
-        const int shift = 8 * p;
-        for (int k = threadIdx.x; k < kWarps * 256; k += kSortThreads) (&wh[0][0])[k] = 0;
-        __syncthreads();
-        uint64_t key[kRounds];
-        uint32_t val[kRounds];
-        unsigned peers[kRounds];
+    int c = 0;
 #pragma unroll
-        for (int r = 0; r < kRounds; ++r) {
-            const int i = base + r * 32 + lane;
-            const bool ok = i < n;
-            key[r] = ok ? kin[i] : 0ull;
-            val[r] = ok ? vin[i] : 0u;
-            const int dg = (int)((key[r] >> shift) & 0xFFu);
-            peers[r] = digit_peers(dg, ok, lane);
-            if (ok && (peers[r] & lt) == 0u) wh[w][dg] += __popc(peers[r]);
-            __syncwarp();
-        }
-        __syncthreads();
-        {
-            const int d = threadIdx.x;
-            int cnt = 0;
+    for (int s = kLen >> 1; s > 0; s >>= 1)
+        if (run[c + s - 1] < lim) c += s;
+    return c + (run[c] < lim ? 1 : 0);
+}
+
+// Merges groups of kLen-key runs (kGroup keys each) of `k` into `ko`.  Padding
+// keys (2^64 - 1, the tail of the tile) are larger than every key and already
+// in the last places of their group: they stay where they are.
+template <int kTile, int kLen, int kGroup>
+__device__ __forceinline__ void merge_padded(const uint64_t *k, const uint16_t *v, uint64_t *ko, uint16_t *vo)
+{
 #pragma unroll
-            for (int k = 0; k < kWarps; ++k) {
-                const int t = wh[k][d];
-                wh[k][d] = cnt;
-                cnt += t;
-            }
-            // exclusive scan of the 256 digit counts: warp scans, then warp totals
-            int incl = cnt;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            if (lane == 31) wtot[w] = incl;
-            dsum[d] = incl - cnt;
-        }
-        __syncthreads();
-        {
-            const int d = threadIdx.x;
-            int off = dsum[d];
-            for (int k = 0; k < w; ++k) off += wtot[k];
+    for (int q = 0; q < kTile / kTileThreads<kTile>; ++q) {
+        const int e = threadIdx.x + q * kTileThreads<kTile>;
+        const uint64_t key = k[e];
+        const int group = e & ~(kGroup - 1), own = (e & (kGroup - 1)) / kLen;
+        int pos = e & (kLen - 1);
 #pragma unroll
-            for (int k = 0; k < kWarps; ++k) wh[k][d] += off;
+        for (int r = 0; r < kGroup / kLen; ++r) {
+            const int c = count_below<kLen>(k + group + r * kLen, key + (r < own ? 1ull : 0ull));
+            pos += r == own ? 0 : c;
         }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kRounds; ++r) {
-            const int i = base + r * 32 + lane;
-            const bool ok = i < n;
-            const int dg = (int)((key[r] >> shift) & 0xFFu);
-            int pos = 0;
-            if (ok) pos = wh[w][dg] + __popc(peers[r] & lt);
-            __syncwarp();
-            if (ok && (peers[r] & lt) == 0u) wh[w][dg] += __popc(peers[r]);
-            __syncwarp();
-            if (ok && pos >= 0 && pos < n) {
-                kout[pos] = key[r];
-                vout[pos] = val[r];
-            }
-        }
-        __syncthreads();  // this pass's output is the next pass's input
+        if (key == ~0ull) pos = e & (kGroup - 1);
+        ko[group + pos] = key;
+        vo[group + pos] = v[e];
     }
+}
+
+template <int kTile>
+__global__ void __launch_bounds__(kTileThreads<kTile>) tile_sort_kernel(const uint64_t *kin, int n, uint64_t *kout,
+                                                                 uint32_t *vout, uint64_t *sample)
+{
+    constexpr int kPer = kTile / kTileThreads<kTile>;
+    extern __shared__ uint64_t sort_shared[];
+    uint64_t *ka = sort_shared, *kb = ka + kTile;
+    uint16_t *va = reinterpret_cast<uint16_t *>(kb + kTile), *vb = va + kTile;
+    const int base = blockIdx.x * kTile, lane = threadIdx.x & 31;
+    uint64_t key[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int e = threadIdx.x + q * kTileThreads<kTile>;
+        key[q] = base + e < n ? kin[base + e] : ~0ull;  // (padding: after every key)
+        ka[e] = key[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {  // runs of 64: 32 keys of the other half of the run, 32 of this warp's
+        const int e = threadIdx.x + q * kTileThreads<kTile>;
+        const uint64_t *run = ka + (e & ~(kRun - 1));
+        const int half = e & 32;
+        const bool pad = key[q] == ~0ull;
+        const uint64_t next = key[q] + (pad ? 0ull : 1ull), other = half ? next : key[q];
+        int rank = 0;
+#pragma unroll 8
+        for (int j = 0; j < 32; ++j) {
+            rank += run[(half ^ 32) + j] < other ? 1 : 0;
+            rank += run[half + j] < (j < lane ? next : key[q]) ? 1 : 0;
+        }
+        if (pad) rank = e & (kRun - 1);  // (a run's padding is its tail already)
+        kb[(e & ~(kRun - 1)) + rank] = key[q];
+        vb[(e & ~(kRun - 1)) + rank] = (uint16_t)e;
+    }
+    __syncthreads();
+    merge_padded<kTile, kRun, kRun2>(kb, vb, ka, va);
+    __syncthreads();
+    if (kTile > kRun2) {
+        merge_padded<kTile, kRun2, kTile>(ka, va, kb, vb);
+        __syncthreads();
+    }
+    const uint64_t *ks = kTile > kRun2 ? kb : ka;
+    const uint16_t *vs = kTile > kRun2 ? vb : va;
+    for (int e = threadIdx.x; e < kTile; e += kTileThreads<kTile>) {
+        if (base + e < n) {
+            kout[base + e] = ks[e];
+            vout[base + e] = (uint32_t)(base + vs[e]);
+        }
+        if (sample && (e & (kSample - 1)) == kSample - 1) sample[(base + e) / kSample] = ks[e];
+    }
+}
+
+// Every key's place among all tiles: its place in its own tile plus, for each
+// other tile, the number of smaller keys there.
+template <int kTile>
+__global__ void __launch_bounds__(1024) rank_scatter_kernel(const uint64_t *__restrict__ kin,
+                                                            const uint32_t *__restrict__ vin,
+                                                            const uint64_t *__restrict__ sample, int n, int tiles,
+                                                            uint64_t *__restrict__ kout, uint32_t *__restrict__ vout,
+                                                            int *status)
+{
+    constexpr int kAtOnce = 8, kPerTile = kTile / kSample;
+    extern __shared__ uint64_t sort_shared[];
+    for (int e = threadIdx.x; e < tiles * kPerTile; e += blockDim.x) sort_shared[e] = sample[e];
+    __syncthreads();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t key = kin[i];
+    const int own = i / kTile;
+    int pos = i - own * kTile;
+    for (int t0 = 0; t0 < tiles; t0 += kAtOnce) {
+        int at[kAtOnce];  // first key of the sampled group that holds the place (n: none)
+#pragma unroll
+        for (int q = 0; q < kAtOnce; ++q) {
+            const int t = t0 + q;
+            at[q] = n;
+            if (t < tiles && t != own) {
+                const int c = count_below<kPerTile>(sort_shared + t * kPerTile, key + (t < own ? 1ull : 0ull));
+                pos += c * kSample;
+                if (c < kPerTile) at[q] = t * kTile + c * kSample;
+            }
+        }
+#pragma unroll
+        for (int s = kSample >> 1; s > 0; s >>= 1) {
+#pragma unroll
+            for (int q = 0; q < kAtOnce; ++q) {  // (fewer than kSample smaller keys in the group)
+                const int p = at[q] + s - 1;
+                if (p < n && __ldg(kin + p) < key + (t0 + q < own ? 1ull : 0ull)) {
+                    at[q] += s;
+                    pos += s;
+                }
+            }
+        }
+    }
+    if (pos >= 0 && pos < n) {
+        kout[pos] = key;
+        vout[pos] = vin[i];
+    } else {
+        atomicOr(status, 4);
+    }
+}
+
+template <int kTile>
+void sort_by_rank(hts_ctx *c)
+{
+    const int n = (int)c->n, tiles = (n + kTile - 1) / kTile;
+    constexpr size_t kShared = 2 * kTile * (sizeof(uint64_t) + sizeof(uint16_t));
+    const size_t samples = sizeof(uint64_t) * (size_t)tiles * (kTile / kSample);
+    if (kShared > 48 * 1024)
+        cudaFuncSetAttribute(tile_sort_kernel<kTile>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kShared);
+    uint64_t *ko = tiles > 1 ? c->keys_alt : c->keys;
+    uint32_t *vo = tiles > 1 ? c->idx_alt : c->idx;
+    uint64_t *sample = tiles > 1 ? reinterpret_cast<uint64_t *>(c->sort_scratch) : nullptr;
+    tile_sort_kernel<kTile><<<tiles, kTileThreads<kTile>, kShared, c->stream>>>(c->keys, n, ko, vo, sample);
+    c->launches += 1;
+    if (tiles == 1) return;
+    static_assert(kRankMax / kSample * 8 + kTile / kSample * 8 <= 48 * 1024, "the sample fits shared memory");
+    const int block = n <= 65536 ? 256 : 1024;  // (every block reads the whole sample)
+    rank_scatter_kernel<kTile><<<(n + block - 1) / block, block, samples, c->stream>>>(
+        c->keys_alt, c->idx_alt, sample, n, tiles, c->keys, c->idx, c->status);
+    c->launches += 1;
 }
 
 }  // namespace
@@ -422,15 +523,15 @@ void launch_sort_pairs(hts_ctx *c)
     const int n = (int)c->n;
     const int tile = tile_keys(n);
     const int tiles = (n + tile - 1) / tile;
-    static_assert(kSmallMax == kSortThreads * 16, "small_sort_kernel<16> covers kSmallMax keys");
-    if (n <= kSmallMax) {  // one block does all eight passes
-        if (n <= kSortThreads * 4)
-            small_sort_kernel<4><<<1, kSortThreads, 0, c->stream>>>(c->keys, c->idx, c->keys_alt, c->idx_alt, n);
-        else if (n <= kSortThreads * 8)
-            small_sort_kernel<8><<<1, kSortThreads, 0, c->stream>>>(c->keys, c->idx, c->keys_alt, c->idx_alt, n);
+    if (n <= kRankMax && c->wait_test == 0) {  // (the wait test needs the look-back)
+        if (n <= kRank512)
+            sort_by_rank<512>(c);
+        else if (n <= kRank1024)
+            sort_by_rank<1024>(c);
+        else if (n <= kRank2048)
+            sort_by_rank<2048>(c);
         else
-            small_sort_kernel<16><<<1, kSortThreads, 0, c->stream>>>(c->keys, c->idx, c->keys_alt, c->idx_alt, n);
-        c->launches += 1;
+            sort_by_rank<4096>(c);
         return;
     }
     // scratch: 2048 ints of digit offsets, 8 tile counters, then the status words
