@@ -136,8 +136,25 @@ __global__ void __launch_bounds__(kBlock) attract_f64_kernel(int n, const int64_
     }
 }
 
-// KL terms in float64 from the float64 positions: per block partial sums of
-// p log p, p log w = -p log1p(d^2) and p, combined in fixed order later.
+// KL terms of one entry in float64 from the float64 positions: adds p log p,
+// p log w = -p log1p(d^2) and p.  The float64 pipe bounds these kernels: about
+// 60 float64 operations with the functions of f64math.cuh (two logarithms, a
+// square root and a division of the library: about 130).
+__device__ __forceinline__ void add_kl_terms(double pv, double2 q, double ai, double2 o, double &a, double &b, double &sp)
+{
+    const double dx = q.x - o.x, dy = q.y - o.y;
+    const double bj = 1.0 - (o.x * o.x + o.y * o.y);
+    const double s = fmax(dx * dx + dy * dy, 1e-300);  // coincident points: log w = 0
+    const double delta = 2.0 * s * reciprocal(ai * bj);
+    double t, rs;
+    sqrt_rsqrt(delta * (delta + 2.0), t, rs);
+    const double d = log1p_pos(delta + t);
+    a += pv * log_pos(pv);
+    b -= pv * log1p_pos(d * d);
+    sp += pv;
+}
+
+// Per block partial sums of the KL terms, combined in fixed order later.
 template <typename VT>
 __global__ void __launch_bounds__(kBlock) kl_terms_kernel(int n, const int64_t *__restrict__ indptr,
                                                           const int32_t *__restrict__ indices,
@@ -154,13 +171,7 @@ __global__ void __launch_bounds__(kBlock) kl_terms_kernel(int n, const int64_t *
             const double pv = (double)vals[e];
             if (!(pv > 0.0)) continue;
             const double2 o = y[indices[e]];
-            double dx = q.x - o.x, dy = q.y - o.y;
-            double bj = 1.0 - (o.x * o.x + o.y * o.y);
-            double delta = 2.0 * (dx * dx + dy * dy) / (ai * bj);
-            double d = log1p(delta + sqrt(delta * (delta + 2.0)));
-            a += pv * log(pv);
-            b -= pv * log1p(d * d);
-            sp += pv;
+            add_kl_terms(pv, q, ai, o, a, b, sp);
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -201,13 +212,7 @@ __global__ void __launch_bounds__(kBlock) kl_rows_kernel(int n, const int64_t *_
         const double pv = (double)vals[e];
         if (!(pv > 0.0)) continue;
         const double2 o = y[indices[e]];
-        double dx = q.x - o.x, dy = q.y - o.y;
-        double bj = 1.0 - (o.x * o.x + o.y * o.y);
-        double delta = 2.0 * (dx * dx + dy * dy) / (ai * bj);
-        double d = log1p(delta + sqrt(delta * (delta + 2.0)));
-        a += pv * log(pv);
-        b -= pv * log1p(d * d);
-        sp += pv;
+        add_kl_terms(pv, q, ai, o, a, b, sp);
     }
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_xor_sync(0xffffffffu, a, o);

@@ -206,13 +206,28 @@ __host__ __device__ __forceinline__ double reciprocal(double x)
     return fma(w0, fma(e, e, e), w0);
 }
 
+// log(1 + m), |m| < 2^-7.99 (5 operations): m + m^2 (-1/2 + m (1/3 + m (-1/4 +
+// m q))), q = 1/5 - m / 6 + m^2 / 7 in float32 (it is worth 2^-32 of the
+// result; the next term of the series 2^-59).
+__host__ __device__ __forceinline__ double log1p_series(double m)
+{
+    const unsigned mh = (unsigned)(bits_of(m) >> 32), ma = mh & 0x7FFFFFFFu;
+    // m as float32 from the top 20 bits of its significand (0 below 2^-123)
+    const float mf = ma < (900u << 20) ? 0.0f : float_of((mh & 0x80000000u) | ((ma << 3) - (896u << 23)));
+    const float q = fmaf(mf, fmaf(mf, 1.0f / 7.0f, -1.0f / 6.0f), 0.2f);
+    const unsigned qb = bits_of(q);
+    const double qd = double_of(((unsigned long long)((qb >> 3) + (896u << 20)) << 32) | (unsigned long long)(qb << 29));
+    double c = fma(m, qd, -0.25);
+    c = fma(m, c, 1.0 / 3.0);
+    c = fma(m, c, -0.5);
+    return fma(m * m, c, m);
+}
+
 // log(1 + g), g >= 0 (11 operations).  z = 1 + g = 2^k v with v rounded to a
 // 1 + j / 128 below 2, m = v r_j - 1 with |m| < 2^-7.99: log z = k log 2 -
 // log r_j + log(1 + m); the first two have an exact sum.  Where k = 0, m =
 // g r + (r - 1) instead, so that small g keeps its digits (r = 1 below
-// g = 2^-8: m = g).  log(1 + m) = m + m^2 (-1/2 + m (1/3 + m (-1/4 + m q))),
-// q = 1/5 - m / 6 + m^2 / 7 in float32 (it is worth 2^-32 of the result; the
-// next term of the series 2^-59).
+// g = 2^-8: m = g).
 __host__ __device__ __forceinline__ double log1p_pos(double g)
 {
     const double z = 1.0 + g;
@@ -230,16 +245,27 @@ __host__ __device__ __forceinline__ double log1p_pos(double g)
     const double a = k == 0 ? g : double_of(zb - ((unsigned long long)(unsigned)k << 52));
     const double b = k == 0 ? r - 1.0 : -1.0;
     const double m = fma(a, r, b);
-    const unsigned mh = (unsigned)(bits_of(m) >> 32), ma = mh & 0x7FFFFFFFu;
-    // m as float32 from the top 20 bits of its significand (0 below 2^-123)
-    const float mf = ma < (900u << 20) ? 0.0f : float_of((mh & 0x80000000u) | ((ma << 3) - (896u << 23)));
-    const float q = fmaf(mf, fmaf(mf, 1.0f / 7.0f, -1.0f / 6.0f), 0.2f);
-    const unsigned qb = bits_of(q);
-    const double qd = double_of(((unsigned long long)((qb >> 3) + (896u << 20)) << 32) | (unsigned long long)(qb << 29));
-    double c = fma(m, qd, -0.25);
-    c = fma(m, c, 1.0 / 3.0);
-    c = fma(m, c, -0.5);
-    return (tt + kh) + (fma(m * m, c, m) + klo);
+    return (tt + kh) + (log1p_series(m) + klo);
+}
+
+// log x, x > 0 normal (8 operations; library outside 2^-127 .. 2^127).
+__host__ __device__ __forceinline__ double log_pos(double x)
+{
+    const unsigned long long xb = bits_of(x);
+    const unsigned xr = (unsigned)(xb >> 32) + 0x1000u;
+    const int k = (int)(xr >> 20) - 1023;
+    if (k < -127 || k > 127) return log(x);
+    const int j = (int)((xr & 0xFFFFFu) >> 13), ka = k < 0 ? -k : k;
+#ifdef __CUDA_ARCH__
+    const double2 tab = __ldg(reinterpret_cast<const double2 *>(kLogTable) + j);
+    const double2 kl = __ldg(reinterpret_cast<const double2 *>(kLn2Table) + ka);
+    const double r = tab.x, tt = tab.y, kh = kl.x, klo = kl.y;
+#else
+    const double r = kLogTable[j].r, tt = kLogTable[j].t, kh = kLn2Table[ka].r, klo = kLn2Table[ka].t;
+#endif
+    const double m = fma(double_of(xb - ((unsigned long long)(long long)k << 52)), r, -1.0);
+    const double lp = log1p_series(m);
+    return k < 0 ? (tt - kh) + (lp - klo) : (tt + kh) + (lp + klo);
 }
 
 #undef HTS_TABLE

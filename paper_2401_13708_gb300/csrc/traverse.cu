@@ -1479,6 +1479,19 @@ __device__ __forceinline__ void exact_ranges(const ExactArgs &A, int i, int &jlo
     cend = min(bhi, cbeg + per * kExactBlock);
 }
 
+// Adds one exact pair (weight 0 unless `take`).
+template <int GF>
+__device__ __forceinline__ void add_exact_f32(float2 qh, float2 ql, float twoil, const PointF &o, bool take, float2 &rxy,
+                                              float2 &rsz)
+{
+    const float2 d = delta2(qh, ql, make_float2(o.xh, o.yh), make_float2(o.xl, o.yl));
+    const float s = fmaf(d.x, d.x, d.y * d.y);
+    const PairF t = pair_terms_f32<GF>(s * twoil * o.il);
+    const float kk = take ? t.rep * o.il : 0.0f;
+    rxy = __ffma2_rn(make_float2(kk, kk), d, rxy);
+    rsz = __ffma2_rn(make_float2(kk, take ? 1.0f : 0.0f), make_float2(s, t.w), rsz);
+}
+
 template <int GF>
 __global__ void __launch_bounds__(kExactBlock) exact_f32_kernel(const PointF *__restrict__ pts, ExactArgs A)
 {
@@ -1496,16 +1509,19 @@ __global__ void __launch_bounds__(kExactBlock) exact_f32_kernel(const PointF *__
         if (j < cend) tile[threadIdx.x] = pts[j];
         __syncthreads();
         const int cnt = min(kExactBlock, cend - base);
-        for (int k = 0; k < cnt; ++k) {
-            const int jj = base + k;
-            if (jj == i || jj < jlo || jj >= jhi) continue;
-            const PointF o = tile[k];
-            const float2 d = delta2(qh, ql, make_float2(o.xh, o.yh), make_float2(o.xl, o.yl));
-            const float s = fmaf(d.x, d.x, d.y * d.y);
-            const PairF t = pair_terms_f32<GF>(s * twoil * o.il);
-            const float kk = t.rep * o.il;
-            rxy = __ffma2_rn(make_float2(kk, kk), d, rxy);
-            rsz = __ffma2_rn(make_float2(kk, 1.0f), make_float2(s, t.w), rsz);
+        // every pair of a full tile off the diagonal and inside the segment
+        // counts: no tests, four pairs in flight (a pair that does not count
+        // is added with weight 0 otherwise)
+        const bool plain = cnt == kExactBlock && !A.seg_of && (base + cnt <= blockIdx.x * kExactBlock ||
+                                                               base >= (blockIdx.x + 1) * kExactBlock);
+        if (plain) {
+#pragma unroll 4
+            for (int k = 0; k < kExactBlock; ++k) add_exact_f32<GF>(qh, ql, twoil, tile[k], true, rxy, rsz);
+        } else {
+            for (int k = 0; k < cnt; ++k) {
+                const int jj = base + k;
+                add_exact_f32<GF>(qh, ql, twoil, tile[k], jj != i && jj >= jlo && jj < jhi, rxy, rsz);
+            }
         }
         __syncthreads();
     }
