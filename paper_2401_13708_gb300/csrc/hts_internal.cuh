@@ -7,7 +7,7 @@
 //   (double2), zi (double), pts32 / pts64 (32-byte point records: position
 //   as float hi/lo pairs or double, and il = 1 / (1 - |y|^2) taken from
 //   float64), apts32 (16-byte records of the float32 attractive sum),
-//   radial (double, split coordinate of the point).
+//   radial (double, |y|^2 of the point).
 // Per point, key order:  keys / idx (uint64 / uint32, sort ping-pong),
 //   spts32 / spts64 (gathered records), terms (Einstein terms, 3 doubles).
 // Binary radix tree over the sorted keys (n - 1 internal nodes): children,

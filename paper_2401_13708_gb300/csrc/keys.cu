@@ -10,32 +10,44 @@
 //   phi^ = atan2 / 2 pi in [0, 1], each quantised to 29 bits and
 //   interleaved (digit l = 2 * radial bit + angular bit of level l, most
 //   significant first), so that the depth-l cell of the equal-length tree is
-//   the top 2l key bits below the 6-bit segment id (bits 58..63).  The float64 steps use explicitly rounded
-//   intrinsics so no fused multiply-add changes a quantised bit.
+//   the top 2l key bits below the 6-bit segment id (bits 58..63).  The bits are
+//   those of the float64 definitions (explicitly rounded, so no fused
+//   multiply-add changes one); float32 pairs decide them where they can.
 #include <cuda_fp16.h>
 
 #include "hts_internal.cuh"
+#include "polar.cuh"
 
 namespace hts {
 namespace {
 
 constexpr int kBlock = 256;
 
-__global__ void init_minmax_kernel(unsigned long long *mm, int nseg)
+__global__ void init_minmax_kernel(unsigned long long *mm, int nseg, unsigned *blocks_done)
 {
     const int s = threadIdx.x;
+    if (s == 0) *blocks_done = 0u;
     if (s < nseg) {
         mm[2 * s] = 0x7FF0000000000000ull;  // +inf
         mm[2 * s + 1] = 0ull;               // +0
     }
 }
 
-// Per point: records and radial coordinate; per segment: the root annulus
-// [min, max] of the radial coordinate (warp-reduced when a warp's points lie
-// in one segment, which is all but the warps straddling a boundary).
+// The radial split coordinate of |y|^2: every operation rounded on its own,
+// and non-decreasing in n2, so that the annulus bounds can be reduced on n2.
+__device__ __forceinline__ double radial_of(double n2, int split_rule)
+{
+    return split_rule == HTS_EQUAL_AREA ? __ddiv_rn(__dadd_rn(1.0, n2), __dsub_rn(1.0, n2)) : __dsqrt_rn(n2);
+}
+
+// Per point: records and |y|^2; per segment: the root annulus [min, max] of the
+// radial coordinate, reduced as |y|^2 (by warps where a warp's points lie in
+// one segment, which is all but the warps straddling a boundary) and converted
+// by the last block.
 __global__ void prep_points_kernel(int n, const double2 *__restrict__ y, int split_rule, PointF *pts32,
                                    PointA *apts32, PointD *pts64, double *radial,
-                                   const unsigned char *__restrict__ seg_of, unsigned long long *mm)
+                                   const unsigned char *__restrict__ seg_of, unsigned long long *mm, int nseg,
+                                   unsigned *blocks_done)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     double c = 0.0;
@@ -58,7 +70,7 @@ __global__ void prep_points_kernel(int n, const double2 *__restrict__ y, int spl
             apts32[i] = PointA{r.xh, r.yh, r.il, lx | (ly << 16)};
         }
         if (pts64) pts64[i] = PointD{p.x, p.y, __ddiv_rn(1.0, __dsub_rn(1.0, n2)), 0.0};
-        c = split_rule == HTS_EQUAL_AREA ? __ddiv_rn(__dadd_rn(1.0, n2), __dsub_rn(1.0, n2)) : __dsqrt_rn(n2);
+        c = n2;
         radial[i] = c;
         if (seg_of) sg = seg_of[i];
     }
@@ -81,6 +93,20 @@ __global__ void prep_points_kernel(int n, const double2 *__restrict__ y, int spl
         atomicMin(&mm[2 * sg], b);
         atomicMax(&mm[2 * sg + 1], b);
     }
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(blocks_done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last && threadIdx.x < nseg) {
+        __threadfence();
+        for (int k = 2 * threadIdx.x; k < 2 * threadIdx.x + 2; ++k) {
+            const unsigned long long v = atomicAdd(&mm[k], 0ull);  // (written by every block's atomics)
+            mm[k] = (unsigned long long)__double_as_longlong(radial_of(__longlong_as_double((long long)v), split_rule));
+        }
+    }
 }
 
 // Spread the low 29 bits of v to the odd/even positions of a 58-bit word.
@@ -100,22 +126,37 @@ __device__ __forceinline__ uint64_t spread_bits(uint64_t v)
 // float64 pipe.
 __device__ __forceinline__ uint64_t quantise(double u) { return quantise_unit(u, kLevels); }
 
-__global__ void make_keys_kernel(int n, const double2 *__restrict__ y, const double *__restrict__ radial,
-                                 const unsigned char *__restrict__ seg_of, const unsigned long long *__restrict__ mm,
-                                 uint64_t *keys, uint32_t *idx)
+// One block: the float32-pair coordinates (polar.cuh) with each segment's
+// annulus prepared once; the float64 definitions where they cannot decide
+// (about 0.1% of the points).
+__global__ void __launch_bounds__(kBlock) make_keys_kernel(int n, const double2 *__restrict__ y,
+                                                           const double *__restrict__ radial,
+                                                           const unsigned char *__restrict__ seg_of,
+                                                           const unsigned long long *__restrict__ mm, int nseg,
+                                                           int split_rule, uint64_t *keys, uint32_t *idx)
 {
+    __shared__ RadialBounds bounds[kMaxSegments];
+    if (threadIdx.x < nseg)
+        bounds[threadIdx.x] = radial_bounds(__longlong_as_double((long long)mm[2 * threadIdx.x]),
+                                            __longlong_as_double((long long)mm[2 * threadIdx.x + 1]));
+    __syncthreads();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int sg = seg_of ? seg_of[i] : 0;
-    double lo = __longlong_as_double((long long)mm[2 * sg]);
-    double hi = __longlong_as_double((long long)mm[2 * sg + 1]);
-    double c = radial[i];
-    double rh = hi > lo ? __ddiv_rn(__dsub_rn(c, lo), __dsub_rn(hi, lo)) : 0.0;
-    double2 p = y[i];
-    double phi = atan2(p.y, p.x);
-    if (phi < 0.0) phi = __dadd_rn(phi, kTwoPi);
-    double ph = __ddiv_rn(phi, kTwoPi);
-    uint64_t qa = quantise(rh), qb = quantise(ph);
+    const double n2 = radial[i];
+    const double2 p = y[i];
+    uint64_t qa, qb;
+    if (!quantise_radius(n2, split_rule == HTS_EQUAL_AREA, bounds[sg], kLevels, qa)) {
+        const double lo = __longlong_as_double((long long)mm[2 * sg]);
+        const double hi = __longlong_as_double((long long)mm[2 * sg + 1]);
+        const double c = radial_of(n2, split_rule);
+        qa = quantise(hi > lo ? __ddiv_rn(__dsub_rn(c, lo), __dsub_rn(hi, lo)) : 0.0);
+    }
+    if (!quantise_angle(p.x, p.y, kLevels, qb)) {
+        double phi = atan2(p.y, p.x);
+        if (phi < 0.0) phi = __dadd_rn(phi, kTwoPi);
+        qb = quantise(__ddiv_rn(phi, kTwoPi));
+    }
     keys[i] = ((uint64_t)sg << kSegShift) | (spread_bits(qa) << 1) | spread_bits(qb);
     idx[i] = (uint32_t)i;
 }
@@ -125,12 +166,13 @@ __global__ void make_keys_kernel(int n, const double2 *__restrict__ y, const dou
 void launch_prep_points(hts_ctx *c)
 {
     int n = (int)c->n;
-    init_minmax_kernel<<<1, kMaxSegments, 0, c->stream>>>(c->minmax, c->nseg);
+    unsigned *blocks_done = reinterpret_cast<unsigned *>(c->minmax + 2 * kMaxSegments + 1);
+    init_minmax_kernel<<<1, kMaxSegments, 0, c->stream>>>(c->minmax, c->nseg, blocks_done);
     bool f32 = c->cfg.precision == HTS_FP32_MIXED;
     prep_points_kernel<<<(n + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
         n, c->y, c->cfg.split_rule, f32 ? c->pts32 : nullptr, f32 ? c->apts32 : nullptr, f32 ? nullptr : c->pts64,
         c->radial,
-        c->nseg > 1 ? c->seg_of : nullptr, c->minmax);
+        c->nseg > 1 ? c->seg_of : nullptr, c->minmax, c->nseg, blocks_done);
     c->launches += 2;
 }
 
@@ -138,7 +180,7 @@ void launch_make_keys(hts_ctx *c)
 {
     int n = (int)c->n;
     make_keys_kernel<<<(n + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
-        n, c->y, c->radial, c->nseg > 1 ? c->seg_of : nullptr, c->minmax, c->keys, c->idx);
+        n, c->y, c->radial, c->nseg > 1 ? c->seg_of : nullptr, c->minmax, c->nseg, c->cfg.split_rule, c->keys, c->idx);
     c->launches += 1;
 }
 

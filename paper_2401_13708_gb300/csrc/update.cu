@@ -186,8 +186,17 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     if (vv > 0.0) {
         // exp map: p (+) tanh(lambda |v| / 2) v / |v|, lambda |v| / 2 = |v| / a;
         // 1 / |v| from one reciprocal square root (no square root and division)
-        const double rn = rsqrt(vv), nv = vv * rn;
-        const double x = nv / a;
+        // float32 mode: from f64math.cuh's seeds (float64 mode keeps the
+        // library's roundings)
+        double rn, nv, x;
+        if (A.rounded) {
+            rn = rsqrt(vv);
+            nv = vv * rn;
+            x = nv / a;
+        } else {
+            sqrt_rsqrt(fmax(vv, 1e-300), nv, rn);
+            x = nv * reciprocal(a);
+        }
         if (A.rounded && x > 2.0) {
             q = long_step(p, v);
         } else {
@@ -196,7 +205,8 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
             const double pu = p.x * ux + p.y * uy;
             const double nu = ux * ux + uy * uy;
             const double ca = 1.0 + 2.0 * pu + nu;
-            const double rden = 1.0 / (1.0 + 2.0 * pu + n2 * nu);
+            const double den = 1.0 + 2.0 * pu + n2 * nu;
+            const double rden = A.rounded ? 1.0 / den : reciprocal(den);
             q.x = (ca * p.x + a * ux) * rden;
             q.y = (ca * p.y + a * uy) * rden;
         }
