@@ -502,6 +502,7 @@ int hts_create(hts_ctx **out, const hts_config *cfg)
     }
     cudaMemset(c->counters, 0, 5 * sizeof(unsigned long long));
     cudaMemset(c->status, 0, sizeof(int));
+    cudaMemset(c->dscal, 0, 8 * sizeof(double));
     *out = c;
     return HTS_OK;
 }

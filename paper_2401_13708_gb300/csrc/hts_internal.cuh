@@ -161,7 +161,7 @@ struct hts_ctx {
     int64_t scan_tmp_len = 0;
     double *red_tmp = nullptr;        // reduction partials
     unsigned long long *minmax = nullptr;  // [2s] min bits, [2s+1] max bits of segment s; then the largest gamma
-    double *dscal = nullptr;          // [0] Z, [1] sum p log p, [2] sum p log w, [3] sum p
+    double *dscal = nullptr;          // [0] Z, [1] sum p log p, [2] sum p log w, [3] sum p; [7] block counter of the Z sum
     int *status = nullptr;
     unsigned long long *counters = nullptr;  // 5: accepted cells, leaf pairs, warp visits, queries, criterion tests
     int *n_nodes = nullptr;          // device scalar: number of tree nodes
@@ -222,7 +222,13 @@ void launch_prep_points(hts_ctx *c);
 void launch_make_keys(hts_ctx *c);
 // sort.cu
 void launch_sort_pairs(hts_ctx *c);
-int scan_exclusive(const int *in, int *out, int64_t len, int *tmp, cudaStream_t s);  // returns kernels launched
+struct CountArgs {  // tree nodes that start at each sorted point: the cells of mask, and the point's own leaf
+    int n;
+    const int *leaf_parent, *pref;
+    const unsigned *mask;
+    int *cnt;       // n + 1 entries, written
+};
+int scan_counts(const CountArgs &counts, int *out, int *tmp, cudaStream_t s);  // returns kernels launched
 int64_t scan_tmp_size(int64_t len);
 size_t sort_status_words(int64_t n);
 // tree.cu

@@ -41,13 +41,13 @@ __device__ __forceinline__ double radial_of(double n2, int split_rule)
 }
 
 // Per point: records and |y|^2; per segment: the root annulus [min, max] of the
-// radial coordinate, reduced as |y|^2 (by warps where a warp's points lie in
-// one segment, which is all but the warps straddling a boundary) and converted
-// by the last block.
-__global__ void prep_points_kernel(int n, const double2 *__restrict__ y, int split_rule, PointF *pts32,
-                                   PointA *apts32, PointD *pts64, double *radial,
-                                   const unsigned char *__restrict__ seg_of, unsigned long long *mm, int nseg,
-                                   unsigned *blocks_done)
+// radial coordinate, reduced as |y|^2 (by warps and blocks where their points lie
+// in one segment, which is all but those straddling a boundary) and converted by
+// the last block.
+__global__ void __launch_bounds__(kBlock) prep_points_kernel(int n, const double2 *__restrict__ y, int split_rule,
+                                                             PointF *pts32, PointA *apts32, PointD *pts64,
+                                                             double *radial, const unsigned char *__restrict__ seg_of,
+                                                             unsigned long long *mm, int nseg, unsigned *blocks_done)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     double c = 0.0;
@@ -74,6 +74,13 @@ __global__ void prep_points_kernel(int n, const double2 *__restrict__ y, int spl
         radial[i] = c;
         if (seg_of) sg = seg_of[i];
     }
+    // the bounds: by warp, then by block where all its points lie in one
+    // segment.  A pair of atomics per warp took most of the kernel at N = 1M
+    // (62,500 on two addresses): 49 us, by block 29 us; 11.3 and 8.6 us at
+    // N = 131,071, no difference below 20,000 points
+    __shared__ unsigned long long wmin[kBlock / 32], wmax[kBlock / 32];
+    __shared__ int wseg[kBlock / 32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned long long b = (unsigned long long)__double_as_longlong(c);
     const int s0 = __shfl_sync(0xffffffffu, sg, 0);
     if (__all_sync(0xffffffffu, !ok || sg == s0)) {
@@ -85,13 +92,39 @@ __global__ void prep_points_kernel(int n, const double2 *__restrict__ y, int spl
             vmin = a < vmin ? a : vmin;
             vmax = z > vmax ? z : vmax;
         }
-        if ((threadIdx.x & 31) == 0 && vmax >= vmin) {
-            atomicMin(&mm[2 * s0], vmin);
-            atomicMax(&mm[2 * s0 + 1], vmax);
+        if (lane == 0) {
+            wmin[w] = vmin;
+            wmax[w] = vmax;
+            wseg[w] = i < n ? s0 : -2;  // (-2: no points)
         }
-    } else if (ok) {
-        atomicMin(&mm[2 * sg], b);
-        atomicMax(&mm[2 * sg + 1], b);
+    } else {
+        if (ok) {
+            atomicMin(&mm[2 * sg], b);
+            atomicMax(&mm[2 * sg + 1], b);
+        }
+        if (lane == 0) wseg[w] = -1;  // done
+    }
+    __syncthreads();
+    if (w == 0) {
+        const int sk = lane < kBlock / 32 ? wseg[lane] : -2;
+        const unsigned have = __ballot_sync(0xffffffffu, sk >= 0);
+        const int sf = __shfl_sync(0xffffffffu, sk, have ? __ffs(have) - 1 : 0);
+        if (__all_sync(0xffffffffu, sk < 0 || sk == sf)) {  // one segment, or nothing left
+            unsigned long long vmin = sk >= 0 ? wmin[lane] : ~0ull, vmax = sk >= 0 ? wmax[lane] : 0ull;
+            for (int o = kBlock / 64; o > 0; o >>= 1) {
+                const unsigned long long a = __shfl_xor_sync(0xffffffffu, vmin, o);
+                const unsigned long long z = __shfl_xor_sync(0xffffffffu, vmax, o);
+                vmin = a < vmin ? a : vmin;
+                vmax = z > vmax ? z : vmax;
+            }
+            if (lane == 0 && have) {
+                atomicMin(&mm[2 * sf], vmin);
+                atomicMax(&mm[2 * sf + 1], vmax);
+            }
+        } else if (sk >= 0) {
+            atomicMin(&mm[2 * sk], wmin[lane]);
+            atomicMax(&mm[2 * sk + 1], wmax[lane]);
+        }
     }
     __shared__ bool last;
     __syncthreads();

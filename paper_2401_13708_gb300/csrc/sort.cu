@@ -261,8 +261,11 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
 
 // ---- exclusive scan --------------------------------------------------------
 
-__global__ void __launch_bounds__(kScanThreads) scan_block_kernel(const int *__restrict__ in, int *out, int64_t len,
-                                                                  int *block_sums)
+// kCount: the input is the number of tree nodes that start at each sorted point
+// (CountArgs), which is also stored.
+template <bool kCount>
+__global__ void __launch_bounds__(kScanThreads) scan_block_kernel(const int *in, const CountArgs counts, int *out,
+                                                                  int64_t len, int *block_sums)
 {
     __shared__ int warp_tot[kScanThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanItems;
@@ -271,7 +274,16 @@ __global__ void __launch_bounds__(kScanThreads) scan_block_kernel(const int *__r
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         int64_t i = base + k;
-        v[k] = i < len ? in[i] : 0;
+        if (kCount) {
+            v[k] = 0;
+            if (i < counts.n) {
+                const bool leaf = counts.n == 1 || quad_level(counts.pref[counts.leaf_parent[i]]) < kLevels;
+                v[k] = __popc(counts.mask[i]) + (leaf ? 1 : 0);
+            }
+            if (i < len) counts.cnt[i] = v[k];
+        } else {
+            v[k] = i < len ? in[i] : 0;
+        }
         local += v[k];
     }
     int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -322,17 +334,30 @@ int64_t scan_tmp_size(int64_t len)
 
 // Exclusive scan of len ints (in and out may alias only if equal).
 // Returns the number of kernels launched.
-int scan_exclusive(const int *in, int *out, int64_t len, int *tmp, cudaStream_t s)
+static int scan_exclusive(const int *in, int *out, int64_t len, int *tmp, cudaStream_t s)
 {
     if (len <= 0) return 0;
     int64_t blocks = (len + kScanBlock - 1) / kScanBlock;
     if (blocks == 1) {
-        scan_block_kernel<<<1, kScanThreads, 0, s>>>(in, out, len, nullptr);
+        scan_block_kernel<false><<<1, kScanThreads, 0, s>>>(in, CountArgs{}, out, len, nullptr);
         return 1;
     }
     int *sums = tmp;
-    scan_block_kernel<<<(unsigned)blocks, kScanThreads, 0, s>>>(in, out, len, sums);
+    scan_block_kernel<false><<<(unsigned)blocks, kScanThreads, 0, s>>>(in, CountArgs{}, out, len, sums);
     int k = scan_exclusive(sums, sums, blocks, tmp + blocks + 1, s);
+    add_offsets_kernel<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(out, len, sums);
+    return k + 2;
+}
+
+// Exclusive scan of the node counts of n sorted points (out: n + 1 entries).
+int scan_counts(const CountArgs &counts, int *out, int *tmp, cudaStream_t s)
+{
+    const int64_t len = (int64_t)counts.n + 1, blocks = (len + kScanBlock - 1) / kScanBlock;
+    int *sums = tmp;
+    scan_block_kernel<true><<<(unsigned)blocks, kScanThreads, 0, s>>>(nullptr, counts, out, len,
+                                                                     blocks > 1 ? sums : nullptr);
+    if (blocks == 1) return 1;
+    const int k = scan_exclusive(sums, sums, blocks, tmp + blocks + 1, s);
     add_offsets_kernel<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(out, len, sums);
     return k + 2;
 }

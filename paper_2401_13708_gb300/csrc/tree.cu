@@ -81,7 +81,13 @@ __global__ void gather_kernel(int n, const uint32_t *__restrict__ idx, const dou
         gb = (unsigned long long)__double_as_longlong(g);
     }
     for (int o = 16; o > 0; o >>= 1) gb = max(gb, __shfl_xor_sync(0xffffffffu, gb, o));
-    if ((threadIdx.x & 31) == 0 && gb) atomicMax(gmax, gb);
+    __shared__ unsigned long long wg[kBlock / 32];
+    if ((threadIdx.x & 31) == 0) wg[threadIdx.x >> 5] = gb;
+    __syncthreads();
+    if (threadIdx.x == 0) {  // one atomic per block: 45 us at N = 1M, 46 with one per warp
+        for (int k = 1; k < kBlock / 32; ++k) gb = max(gb, wg[k]);
+        if (gb) atomicMax(gmax, gb);
+    }
 }
 
 __device__ __forceinline__ int prefix_len(const uint64_t *__restrict__ keys, int n, int i, int j)
@@ -192,12 +198,12 @@ __device__ __forceinline__ double fx_to_double(fx_t v, int E)
 }
 
 // One block scans kScanB consecutive elements: out[i] = exclusive prefix within
-// the block, tot[block] = block total.  Input: float64 terms (3 per point,
-// converted with the exponent from *gmax) when `terms` is given, otherwise
-// FX3 values.
+// the block, tot[block] = block total (a grid of one block also writes it to
+// *grand).  Input: float64 terms (3 per point, converted with the exponent from
+// *gmax) when `terms` is given, otherwise FX3 values (in and out may be the same).
 __global__ void __launch_bounds__(kScanT) fx_scan_block_kernel(int len, const double *__restrict__ terms,
                                                               const unsigned long long *__restrict__ gmax, int n,
-                                                              const FX3 *__restrict__ in, FX3 *out, FX3 *tot)
+                                                              const FX3 *in, FX3 *out, FX3 *tot, FX3 *grand)
 {
     __shared__ FX3 wsum[kScanT / 32];
     const int E = terms ? fx_exponent(*gmax, n) : 0;
@@ -238,7 +244,10 @@ __global__ void __launch_bounds__(kScanT) fx_scan_block_kernel(int len, const do
         if (i < len) out[i] = run;
         run = fx3_add(run, v[k]);
     }
-    if (threadIdx.x == kScanT - 1) tot[blockIdx.x] = run;
+    if (threadIdx.x == kScanT - 1) {
+        tot[blockIdx.x] = run;
+        if (gridDim.x == 1) *grand = run;
+    }
 }
 
 __global__ void fx_scan_add_kernel(int len, FX3 *out, const FX3 *__restrict__ off)
@@ -247,22 +256,24 @@ __global__ void fx_scan_add_kernel(int len, FX3 *out, const FX3 *__restrict__ of
     if (i < len) out[i] = fx3_add(off[i / kScanB], out[i]);
 }
 
-// Exclusive scan of len elements into out[0 .. len-1]; the grand total goes to
-// *total.  tmp holds the block totals of every recursion level.
+// Exclusive scan of len elements: out[i] is the prefix within i's block of
+// kScanB, tmp[i / kScanB] (len > kScanB) the prefix of the block, *total the grand
+// total.  emit adds the two: a pass over out of its own would read and write the
+// 48 bytes per point once more, and is one launch more at every size.  The scan
+// takes 45 us at N = 1M (72 MB moved).  tmp holds the block totals of every level.
 void fx_scan(int len, const double *terms, const unsigned long long *gmax, int n, const FX3 *in, FX3 *out,
              FX3 *total, FX3 *tmp, cudaStream_t s, int64_t *launches)
 {
     const int blocks = (len + kScanB - 1) / kScanB;
     FX3 *tot = tmp;
-    fx_scan_block_kernel<<<blocks, kScanT, 0, s>>>(len, terms, gmax, n, in, out, tot);
+    fx_scan_block_kernel<<<blocks, kScanT, 0, s>>>(len, terms, gmax, n, in, out, tot, total);
     *launches += 1;
-    if (blocks == 1) {
-        cudaMemcpyAsync(total, tot, sizeof(FX3), cudaMemcpyDeviceToDevice, s);
-        return;
-    }
+    if (blocks == 1) return;
     fx_scan(blocks, nullptr, nullptr, 0, tot, tot, total, tmp + blocks, s, launches);
-    fx_scan_add_kernel<<<(len + 255) / 256, 256, 0, s>>>(len, out, tot);
-    *launches += 1;
+    if (blocks > kScanB) {
+        fx_scan_add_kernel<<<(blocks + 255) / 256, 256, 0, s>>>(blocks, tot, tmp + blocks);
+        *launches += 1;
+    }
 }
 
 // Quad levels present among the cells whose first sorted point is p, one bit
@@ -280,18 +291,6 @@ __global__ void quad_mark_kernel(int n, const int *__restrict__ parent, const in
         int q = lv > pl;
         quad[k] = q;
         if (q) atomicOr(&mask[lo_arr[k]], 1u << lv);
-    }
-}
-
-__global__ void count_kernel(int n, const int *__restrict__ leaf_parent, const int *__restrict__ pref,
-                             const unsigned *__restrict__ mask, int *cnt)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) {
-        bool leaf = n == 1 || quad_level(pref[leaf_parent[k]]) < kLevels;
-        cnt[k] = __popc(mask[k]) + (leaf ? 1 : 0);
-    } else if (k == n) {
-        cnt[n] = 0;
     }
 }
 
@@ -356,18 +355,24 @@ __device__ __forceinline__ float acosh1p_f32(float delta)
     return delta < 0.1f ? t * fs : __logf(1.0f + delta + t);
 }
 
+// (float)v, rounded with integer operations where v is in their range.
+__device__ __forceinline__ float to_f32(double v)
+{
+    float hi, lo;
+    split_f32(v, hi, lo);
+    return hi;
+}
+
 __device__ float cell_threshold_f32(double lo, double hi, uint64_t a, int ell, int rule, double theta)
 {
-    double scale = ldexp(1.0, -ell);
-    double span = hi - lo;
-    double c0 = lo + span * ((double)a * scale);
-    double c1 = lo + span * ((double)(a + 1) * scale);
-    double dc = span * scale;
+    const double dc = (hi - lo) * pow2(-ell);  // the power of two is exact: the bounds are lo + span (a 2^-ell)
+    double c0 = fma(dc, (double)(int)a, lo);
+    double c1 = fma(dc, (double)(int)(a + 1), lo);
     double r0 = radius_of(c0, rule), r1 = radius_of(c1, rule);
     double dr = rule == HTS_EQUAL_AREA ? (r0 + r1 > 0.0 ? 2.0 * dc / ((c0 + 1.0) * (c1 + 1.0) * (r0 + r1)) : 0.0)
                                        : dc;
-    const float a0 = (float)((1.0 - r0) * (1.0 + r0)), a1 = (float)((1.0 - r1) * (1.0 + r1));
-    const float f0 = (float)r0, f1 = (float)r1, fdr = (float)dr;
+    const float a0 = to_f32((1.0 - r0) * (1.0 + r0)), a1 = to_f32((1.0 - r1) * (1.0 + r1));
+    const float f0 = to_f32(r0), f1 = to_f32(r1), fdr = to_f32(dr);
     const float sh = sinpif(ldexpf(1.0f, -ell));  // sin(dphi / 2), dphi = 2 pi 2^-ell: relative accuracy
     const float sh2 = sh * sh;
     const float diag = acosh1p_f32(2.0f * (fdr * fdr + 4.0f * f0 * f1 * sh2) / (a0 * a1));
@@ -406,7 +411,8 @@ struct EmitArgs {
     const int *left, *parent, *leaf_parent, *lo_arr, *hi_arr, *pref, *quad, *pre;
     int *cnt;
     const unsigned *mask;
-    const FX3 *prefix;  // n + 1 exclusive prefix sums of the Einstein terms (fixed point)
+    const FX3 *prefix;  // n + 1 exclusive prefix sums of the Einstein terms (fixed point), within blocks of kScanB
+    const FX3 *block_prefix;  // and before each block (nullptr: one block)
     const unsigned long long *gmax;  // largest gamma (bits): the fixed-point exponent
     const unsigned long long *mm;
     NodeF *nodes32;
@@ -415,6 +421,13 @@ struct EmitArgs {
     int capacity;
     int *status;
 };
+
+// Prefix sum before sorted point p (p = n: of all points).
+__device__ __forceinline__ FX3 prefix_at(const EmitArgs &A, int p)
+{
+    const FX3 v = A.prefix[p];
+    return A.block_prefix && p < A.n ? fx3_add(A.block_prefix[p / kScanB], v) : v;
+}
 
 __global__ void emit_kernel(EmitArgs A)
 {
@@ -430,7 +443,7 @@ __global__ void emit_kernel(EmitArgs A)
         int rank = __popc(A.mask[lo] & ((1u << ell) - 1u));  // shallower cells starting at lo
         int pos = A.pre[lo] + rank;
         int skip = A.pre[hi + 1];
-        const FX3 p1 = A.prefix[hi + 1], p0 = A.prefix[lo];
+        const FX3 p1 = prefix_at(A, hi + 1), p0 = prefix_at(A, lo);
         double cx, cy, beta;
         if (A.nodes64 || A.ex.depth) {  // float64 walk / export: the oracle's correctly rounded steps
             const int E = fx_exponent(*A.gmax, n);
@@ -605,7 +618,7 @@ void launch_build_tree(hts_ctx *c, double theta, const TreeExport *ex)
     cudaStreamWaitEvent(ts, c->tev_fork, 0);
     gather_kernel<<<gp, kBlock, 0, ts>>>(n, c->idx, c->y, c->pts32, c->pts64, f32 ? c->spts32 : nullptr,
                                          f32 ? nullptr : c->spts64, c->terms, gmax, (!f32 || ex) ? 1 : 0);
-    c->launches += 4;  // gather, quad_mark, count, emit
+    c->launches += 3;  // gather, quad_mark, emit
     if (n > 1)
         fx_scan(n, c->terms, gmax, n, nullptr, prefix, prefix + n, reinterpret_cast<FX3 *>(c->red_tmp), ts,
                 &c->launches);
@@ -618,8 +631,7 @@ void launch_build_tree(hts_ctx *c, double theta, const TreeExport *ex)
         quad_mark_kernel<<<gp, kBlock, 0, s>>>(n, c->bn_parent, c->leaf_parent, c->bn_lo, c->bn_pref, c->bn_quad,
                                                mask);
     }
-    count_kernel<<<(n + 1 + kBlock - 1) / kBlock, kBlock, 0, s>>>(n, c->leaf_parent, c->bn_pref, mask, c->cnt);
-    c->launches += scan_exclusive(c->cnt, c->pre, (int64_t)n + 1, c->scan_tmp, s);
+    c->launches += scan_counts(CountArgs{n, c->leaf_parent, c->bn_pref, mask, c->cnt}, c->pre, c->scan_tmp, s);
     cudaStreamWaitEvent(s, c->tev_join, 0);
     EmitArgs A;
     A.n = n;
@@ -641,6 +653,7 @@ void launch_build_tree(hts_ctx *c, double theta, const TreeExport *ex)
     A.pre = c->pre;
     A.mask = mask;
     A.prefix = prefix;
+    A.block_prefix = n > kScanB ? reinterpret_cast<const FX3 *>(c->red_tmp) : nullptr;
     A.mm = c->minmax;
     A.gmax = gmax;
     A.nodes32 = c->nodes32;

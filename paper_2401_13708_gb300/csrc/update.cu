@@ -1,7 +1,7 @@
 // update.cu -- Z, the gradient and the Riemannian step, all in float64.
 //
-// reduce_z   Z = sum_i Z_i in a fixed order (256 fixed block partials, then
-//            one block), so the value is reproducible.
+// reduce_z   Z = sum_i Z_i in a fixed order (256 fixed block partials, added by
+//            the last block), so the value is reproducible.
 // update     g_i = 4 (exag F_attr,i - F_rep,i / Z)  (Eq. KlGradientHyperbolicSplit
 //            with the exaggeration of Sec. 5.1), then
 //              r_i = lambda_i^-metric_pow g_i  ("product of lambda^-1 with the
@@ -26,13 +26,16 @@ constexpr int kBlock = 256;
 // sort position out of range (4), a bounded look-back wait ran out (128)
 constexpr int kStepBlockingStatus = 2 | 4 | 128;
 
-// Fixed-shape two-pass sum: kRedBlocks blocks reduce grid-strided slices,
-// one block adds the partials in order -- reproducible for a given n.
+// Fixed-shape sum: kRedBlocks blocks reduce grid-strided slices, the last one to
+// finish adds the partials in order -- reproducible for a given n.
 constexpr int kRedBlocks = 256;
 
-__global__ void __launch_bounds__(kBlock) partial_sum_kernel(int n, const double *__restrict__ v, double *partial)
+__global__ void __launch_bounds__(kBlock) sum_kernel(int n, const double *__restrict__ v, double *partial, double *out,
+                                                     unsigned *blocks_done)
 {
+    static_assert(kBlock == kRedBlocks, "the last block adds one partial per thread");
     __shared__ double sh[kBlock];
+    __shared__ bool last;
     double a = 0;
     for (int k = blockIdx.x * kBlock + threadIdx.x; k < n; k += kRedBlocks * kBlock) a += v[k];
     sh[threadIdx.x] = a;
@@ -41,19 +44,26 @@ __global__ void __launch_bounds__(kBlock) partial_sum_kernel(int n, const double
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-__global__ void __launch_bounds__(kRedBlocks) final_sum_kernel(const double *__restrict__ partial, double *out)
-{
-    __shared__ double sh[kRedBlocks];
-    sh[threadIdx.x] = partial[threadIdx.x];
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = sh[0];
+        __threadfence();
+        last = atomicAdd(blocks_done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    // the last block to finish adds the partials (in a fixed order) and leaves
+    // the counter at zero for the next sum
+    __threadfence();
+    sh[threadIdx.x] = __ldcg(partial + threadIdx.x);
     __syncthreads();
     for (int s = kRedBlocks / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = sh[0];
+    if (threadIdx.x == 0) {
+        *out = sh[0];
+        *blocks_done = 0u;
+    }
 }
 
 // Per-segment sum of v over [off[s], off[s+1]), one block per segment.
@@ -243,9 +253,9 @@ void launch_reduce_z(hts_ctx *c)
         return;
     }
     double *partial = c->red_tmp;  // >= kRedBlocks doubles
-    partial_sum_kernel<<<kRedBlocks, kBlock, 0, c->stream>>>((int)c->n, c->zi, partial);
-    final_sum_kernel<<<1, kRedBlocks, 0, c->stream>>>(partial, c->dscal);
-    c->launches += 2;
+    sum_kernel<<<kRedBlocks, kBlock, 0, c->stream>>>((int)c->n, c->zi, partial, c->dscal,
+                                                     reinterpret_cast<unsigned *>(c->dscal + 7));
+    c->launches += 1;
 }
 
 void launch_update(hts_ctx *c, double exag, double lr, double mom, double2 *g_out, int do_step)
