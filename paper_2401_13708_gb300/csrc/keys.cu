@@ -23,10 +23,14 @@ namespace {
 
 constexpr int kBlock = 256;
 
-__global__ void init_minmax_kernel(unsigned long long *mm, int nseg, unsigned *blocks_done)
+// (gmax: the largest gamma of the tree that the keys lead to, collected by gather)
+__global__ void init_minmax_kernel(unsigned long long *mm, int nseg, unsigned long long *gmax, unsigned *blocks_done)
 {
     const int s = threadIdx.x;
-    if (s == 0) *blocks_done = 0u;
+    if (s == 0) {
+        *gmax = 0ull;
+        *blocks_done = 0u;
+    }
     if (s < nseg) {
         mm[2 * s] = 0x7FF0000000000000ull;  // +inf
         mm[2 * s + 1] = 0ull;               // +0
@@ -166,7 +170,8 @@ __global__ void __launch_bounds__(kBlock) make_keys_kernel(int n, const double2 
                                                            const double *__restrict__ radial,
                                                            const unsigned char *__restrict__ seg_of,
                                                            const unsigned long long *__restrict__ mm, int nseg,
-                                                           int split_rule, uint64_t *keys, uint32_t *idx)
+                                                           int split_rule, uint64_t *keys, uint32_t *idx,
+                                                           unsigned *mask)
 {
     __shared__ RadialBounds bounds[kMaxSegments];
     if (threadIdx.x < nseg)
@@ -192,6 +197,7 @@ __global__ void __launch_bounds__(kBlock) make_keys_kernel(int n, const double2 
     }
     keys[i] = ((uint64_t)sg << kSegShift) | (spread_bits(qa) << 1) | spread_bits(qb);
     idx[i] = (uint32_t)i;
+    mask[i] = 0u;  // the tree's quad levels, set by quad_mark: a memset node less
 }
 
 }  // namespace
@@ -200,7 +206,7 @@ void launch_prep_points(hts_ctx *c)
 {
     int n = (int)c->n;
     unsigned *blocks_done = reinterpret_cast<unsigned *>(c->minmax + 2 * kMaxSegments + 1);
-    init_minmax_kernel<<<1, kMaxSegments, 0, c->stream>>>(c->minmax, c->nseg, blocks_done);
+    init_minmax_kernel<<<1, kMaxSegments, 0, c->stream>>>(c->minmax, c->nseg, c->minmax + 2 * kMaxSegments, blocks_done);
     bool f32 = c->cfg.precision == HTS_FP32_MIXED;
     prep_points_kernel<<<(n + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
         n, c->y, c->cfg.split_rule, f32 ? c->pts32 : nullptr, f32 ? c->apts32 : nullptr, f32 ? nullptr : c->pts64,
@@ -213,7 +219,8 @@ void launch_make_keys(hts_ctx *c)
 {
     int n = (int)c->n;
     make_keys_kernel<<<(n + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(
-        n, c->y, c->radial, c->nseg > 1 ? c->seg_of : nullptr, c->minmax, c->nseg, c->cfg.split_rule, c->keys, c->idx);
+        n, c->y, c->radial, c->nseg > 1 ? c->seg_of : nullptr, c->minmax, c->nseg, c->cfg.split_rule, c->keys, c->idx,
+        reinterpret_cast<unsigned *>(c->bn_flag));
     c->launches += 1;
 }
 

@@ -607,8 +607,7 @@ void launch_build_tree(hts_ctx *c, double theta, const TreeExport *ex)
     unsigned long long *gmax = c->minmax + 2 * kMaxSegments;
     FX3 *prefix = reinterpret_cast<FX3 *>(c->bn_sum);  // n + 1 entries
     unsigned *mask = reinterpret_cast<unsigned *>(c->bn_flag);
-    cudaMemsetAsync(gmax, 0, sizeof(unsigned long long), s);
-    cudaMemsetAsync(mask, 0, sizeof(unsigned) * (size_t)n, s);
+    // (gmax and mask were zeroed with the annulus bounds and the keys)
     // two independent chains, joined before emit: on the side stream the
     // sorted point records and the fixed-point prefix sums of the Einstein
     // terms; here the radix tree, the quad-level marks and the node layout
