@@ -324,7 +324,8 @@ HTS_API int hts_get_tuning(const hts_ctx *ctx, int *tuning);
 HTS_API int hts_measure_peaks(int device, double *out3);
 
 /* Test of the bounded device-side waits (no counterpart in the paper).  The
- * one-sweep sort passes (problems of more than 4096 points) wait, per tile,
+ * one-sweep sort passes (problems of more than 150,000 points, and of more than
+ * 4096 while this test is on) wait, per tile,
  * for the digit counts of earlier tiles; every such wait gives up after a
  * bounded number of polls (~0.3 s), sets a status bit and writes no key out
  * of range, so that a lost publication can never hang the GPU.  With

@@ -1,9 +1,8 @@
 // api.cu -- the C ABI of libhts (declared in include/hts.h).
 //
 // One iteration (hts_step) queues, on the context's stream:
-//   prep_points -> make_keys -> sort (8 passes) -> build_tree -> walk
-//   -> attract -> reduce_z -> update
-// or, for theta == 0, prep_points -> exact -> attract -> reduce_z -> update.
+//   prep_points -> make_keys -> sort -> build_tree -> walk -> reduce_z -> update
+// with attract beside the tree build and the walk, or, for theta == 0, prep_points -> exact -> attract -> reduce_z -> update.
 // Nothing is allocated and nothing is copied to the host inside the loop;
 // the status word is read once after the last iteration.
 #include <math.h>

@@ -161,7 +161,8 @@ struct hts_ctx {
     int64_t scan_tmp_len = 0;
     double *red_tmp = nullptr;        // reduction partials
     unsigned long long *minmax = nullptr;  // [2s] min bits, [2s+1] max bits of segment s; then the largest gamma
-    double *dscal = nullptr;          // [0] Z, [1] sum p log p, [2] sum p log w, [3] sum p; [7] block counter of the Z sum
+    // [0] Z, [1] sum p log p, [2] sum p log w, [3] sum p; [7] block counter of the Z sum (0 between sums)
+    double *dscal = nullptr;
     int *status = nullptr;
     unsigned long long *counters = nullptr;  // 5: accepted cells, leaf pairs, warp visits, queries, criterion tests
     int *n_nodes = nullptr;          // device scalar: number of tree nodes
@@ -239,8 +240,8 @@ void launch_exact(hts_ctx *c);
 // j-chunks of the exact kernel for n points (1 when the i-blocks alone fill
 // the GPU); the partial sums take exact_split(n) * n double4 when it is > 1
 int exact_split(int64_t n);
-// split walk: buffer capacity (frontier entries) for n points, the depth used,
-// and the bytes of the frontier table
+// split walk: buffer capacity (subtrees) for n points, the depth used,
+// and the bytes of the tables of the cuts
 int walk_split_capacity(int64_t n);
 int walk_split_depth(int64_t n, int want, bool fp64);
 size_t walk_split_frontier_bytes();

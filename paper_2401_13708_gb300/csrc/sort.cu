@@ -45,6 +45,7 @@ namespace {
 //   131,071                               14.1 + 48.2  31.7 + 26.9  60.8
 //   262,144                               14.1 + 177   31.8 + 95.5  76.4
 constexpr int64_t kRankMax = 150000, kRank512 = 8192, kRank1024 = 32768, kRank2048 = 90000;
+constexpr int kWaitTestFrom = 4096;  // (hts_set_wait_test)
 constexpr int kMinTile = 1024;     // one-sweep tiles hold 1024, 2048, 4096 or 8192 keys (tile_keys)
 constexpr int kSortThreads = 256;
 constexpr int kScanThreads = 1024;
@@ -548,7 +549,8 @@ void launch_sort_pairs(hts_ctx *c)
     const int n = (int)c->n;
     const int tile = tile_keys(n);
     const int tiles = (n + tile - 1) / tile;
-    if (n <= kRankMax && c->wait_test == 0) {  // (the wait test needs the look-back)
+    // (the wait test is about the look-back, which up to kWaitTestFrom keys is never asked for)
+    if (n <= kRankMax && (c->wait_test == 0 || n <= kWaitTestFrom)) {
         if (n <= kRank512)
             sort_by_rank<512>(c);
         else if (n <= kRank1024)

@@ -18,12 +18,16 @@
 // walk; the warp visits the union of the 32 walks.  Node loads are
 // warp-uniform (one sector, broadcast) and stay in L1/L2.
 //
+// Two forms: direct (walk_*: the terms are added as the cursor goes) and listed
+// (list_*: many warps per chunk, one per subtree, write down which interactions
+// each lane takes; sum_*: the terms of the listed ones, in the order of the walk
+// in float32).  launch_walk chooses by size and precision.
+//
 // Per lane the pair term is reduced to a scalar times (Delta, s) and a w
 // for Z (see pair_terms_* in hts_internal.cuh); the result per point is
 //   F_rep,i = 4 il_i (R_Delta + il_i R_s y_i),   Z_i = sum N w,
 // written to the point's original index.
 #include <limits.h>
-
 
 #include <algorithm>
 
@@ -33,10 +37,7 @@ namespace hts {
 namespace {
 
 constexpr int kWalkBlock = 256;
-#ifndef LB
-#define LB 128
-#endif
-constexpr int kListBlock = LB;
+constexpr int kListBlock = 128;
 constexpr int kExactBlock = 64;
 
 // One node, read through the non-coherent path: a single 256-bit load (the
@@ -1596,19 +1597,13 @@ int walk_split_capacity(int64_t n)
 // 40,000 / 100,000 warps 183 / 142 / 205 us).  In float64 the pair terms are
 // most of the walk and the listed ones fill the float64 pipe better (N =
 // 70,000: 8.2 ms direct, 0.5 + 7.3 ms listed), so the limit is the lists' size.
-#ifndef LW
-#define LW 40000
-#endif
-#ifndef LMAX
-#define LMAX 128
-#endif
-constexpr int64_t kListWarps = LW;
+constexpr int64_t kListWarps = 40000, kListTargetMax = 128;
 constexpr int64_t kListMaxN = 1 << 15, kListMaxN64 = 1 << 18;
 
 static int list_target(int64_t n)
 {
     const int64_t chunks = std::max<int64_t>((n + 31) / 32, 1);
-    return (int)std::max<int64_t>(2, std::min<int64_t>(kListWarps / chunks, LMAX));
+    return (int)std::max<int64_t>(2, std::min<int64_t>(kListWarps / chunks, kListTargetMax));
 }
 
 // First pages per chunk: the cap of the cut into units (a cut by point counts

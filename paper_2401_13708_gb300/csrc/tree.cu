@@ -20,6 +20,7 @@
 //                 exactly (E >= ~90 for 1M points within 1 - 1e-4 of the rim);
 //                 smaller ones are truncated at 2^-E.  Integer adds keep the
 //                 scan off the float64 pipe, which is narrow on this GPU.
+//                 (Stored within blocks and per block; emit adds the two.)
 //  4. quad nodes  a binary node is a quadtree cell iff its quad level
 //                 floor(prefix_bits / 2) exceeds its parent's; that is the
 //                 deepest cell of a chain of one-child cells (chains collapse:

@@ -24,3 +24,17 @@ def test_tree_of_the_sorted_keys(n, ties):
     o = oracle.tree_export(y, 0, which=1)
     for k in ("depth", "prefix", "count", "first"):
         assert np.array_equal(g[k], o[k]), k
+
+
+@pytest.mark.parametrize("n", [2000, 4096])
+def test_small_sorts_wait_for_nothing(n):
+    """The wait test's limit applies to sorts of more than 4096 keys only."""
+    y = inputs.spread_embedding(np.arange(n) % 37, 3, rho_hi=8.0)
+    with HyperbolicTSNE(precision="fp32") as t:
+        t.set_P(np.zeros(n + 1, np.int64), np.zeros(0, np.int32), np.zeros(0, np.float32))
+        t.set_Y(y)
+        g, _ = t.grad(0.5)
+        t._check(t._lib.hts_set_wait_test(t._ctx, 8))
+        h, _ = t.grad(0.5)
+        t._check(t._lib.hts_set_wait_test(t._ctx, 0))
+    assert np.array_equal(g, h)
