@@ -88,7 +88,8 @@ struct UpdateArgs {
     double2 *y, *vel, *gains;
     const double2 *fattr, *frep;
     const double *Z;
-    double exag, lr, mom, eps;
+    double exag4, lr, mom, eps;  // 4 x the exaggeration; the learning rate x 2^-metric_pow
+    double lim2;                 // (1 - eps / 2)^2
     int metric_pow, use_gains, do_step;
     int rounded;  // float64 mode: |y|^2 and long steps with every operation rounded on its own
     double2 *g_out;
@@ -136,6 +137,22 @@ __device__ __noinline__ double2 long_step(double2 p, double2 v)
                         __ddiv_rn(__dadd_rn(__dmul_rn(ca, p.y), __dmul_rn(cb, uy)), den));
 }
 
+// Comparisons by bit patterns, off the float64 pipe.
+__device__ __forceinline__ bool positive(double x)  // x > 0 (not NaN)
+{
+    return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7FF0000000000000ull;
+}
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7FFFFFFF) < 0x7FF00000; }
+__device__ __forceinline__ bool not_below(double x, double lim)  // x >= lim, for x, lim >= 0 (x not NaN)
+{
+    const long long b = __double_as_longlong(x);
+    return b >= __double_as_longlong(lim) && b <= 0x7FF0000000000000ll;
+}
+
+// Bound by the float64 pipe (81% busy: ~80 operations a point at two lanes a
+// cycle per SM, N = 1M 115 us; its 96 bytes a point would take 15 us), so
+// factors that are powers of two are folded into the arguments (the same bits)
+// and tests are made on bit patterns: 142 us with 15 operations more.
 __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
 {
     __shared__ double s_invz;
@@ -143,22 +160,22 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     if (!A.seg_of) {  // one problem: 1 / Z once per block (float64 division is costly here)
         if (threadIdx.x == 0) {
             const double Z0 = A.Z[0];
-            s_invz = Z0 > 0.0 ? 1.0 / Z0 : 0.0;
+            s_invz = Z0 > 0.0 ? 4.0 * (1.0 / Z0) : 0.0;
         }
         __syncthreads();
     }
     if (i >= A.n) return;
     const int sg = A.seg_of ? A.seg_of[i] : 0;
-    double invZ;
+    double invZ4;  // 4 / Z
     if (A.seg_of) {
         const double Z = A.Z[sg];
-        invZ = Z > 0.0 ? 1.0 / Z : 0.0;
+        invZ4 = Z > 0.0 ? 4.0 * (1.0 / Z) : 0.0;
     } else {
-        invZ = s_invz;
+        invZ4 = s_invz;
     }
     const double2 fa = A.fattr[i], fr = A.frep[i];
-    double gx = 4.0 * (A.exag * fa.x - fr.x * invZ);
-    double gy = 4.0 * (A.exag * fa.y - fr.y * invZ);
+    double gx = A.exag4 * fa.x - fr.x * invZ4;
+    double gy = A.exag4 * fa.y - fr.y * invZ4;
     double2 p = A.y[i];
     const double n2 = A.rounded ? __dadd_rn(__dmul_rn(p.x, p.x), __dmul_rn(p.y, p.y)) : p.x * p.x + p.y * p.y;
     if (A.xsq) {  // CO-SNE: lambda1 g_KL - (4 lambda2 / n)(|x|^2 - |y|^2) y
@@ -175,9 +192,11 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     if (*(volatile const int *)A.status & kStepBlockingStatus) return;
     double2 v = A.vel[i];
     const double a = 1.0 - n2;  // 2 / lambda (Eq. PoincareMetric)
-    const double hl = 0.5 * a;  // 1 / lambda
-    const double sc = A.metric_pow == 2 ? hl * hl : hl;
-    double kx = 1.0, ky = 1.0;
+    // the metric's factor lambda^-metric_pow is (a / 2)^metric_pow; the power of
+    // two is in A.lr
+    const double sc = A.metric_pow == 2 ? a * a : a;
+    const double lr = A.seg_of ? A.lr * A.seg_lr[sg] : A.lr;
+    double lx = lr, ly = lr;
     if (A.use_gains) {
         double2 gn = A.gains[i];
         gn.x = ((gx > 0.0) == (v.x > 0.0)) ? gn.x * 0.8 : gn.x + 0.2;
@@ -185,15 +204,14 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
         gn.x = fmax(gn.x, 0.01);
         gn.y = fmax(gn.y, 0.01);
         A.gains[i] = gn;
-        kx = gn.x;
-        ky = gn.y;
+        lx = lr * gn.x;
+        ly = lr * gn.y;
     }
-    const double lr = A.seg_of ? A.lr * A.seg_lr[sg] : A.lr;
-    v.x = A.mom * v.x - lr * kx * (gx * sc);
-    v.y = A.mom * v.y - lr * ky * (gy * sc);
+    v.x = A.mom * v.x - lx * (gx * sc);
+    v.y = A.mom * v.y - ly * (gy * sc);
     const double vv = v.x * v.x + v.y * v.y;
     double2 q = p;
-    if (vv > 0.0) {
+    if (positive(vv)) {
         // exp map: p (+) tanh(lambda |v| / 2) v / |v|, lambda |v| / 2 = |v| / a;
         // 1 / |v| from one reciprocal square root (no square root and division)
         // float32 mode: from f64math.cuh's seeds (float64 mode keeps the
@@ -204,7 +222,7 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
             nv = vv * rn;
             x = nv / a;
         } else {
-            sqrt_rsqrt(fmax(vv, 1e-300), nv, rn);
+            sqrt_rsqrt(not_below(vv, 1e-300) ? vv : 1e-300, nv, rn);
             x = nv * reciprocal(a);
         }
         if (A.rounded && x > 2.0) {
@@ -222,13 +240,12 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
         }
     }
     const double q2 = q.x * q.x + q.y * q.y;
-    const double lim = 1.0 - A.eps / 2.0;
-    if (q2 >= lim * lim) {  // |q| >= 1 - eps/2 (Eq. HyperbolicProjection): back to radius 1 - eps
+    if (not_below(q2, A.lim2)) {  // |q| >= 1 - eps/2 (Eq. HyperbolicProjection): back to radius 1 - eps
         const double f = (1.0 - A.eps) / sqrt(q2);
         q.x *= f;
         q.y *= f;
     }
-    if (!isfinite(q.x) || !isfinite(q.y) || !isfinite(v.x) || !isfinite(v.y)) atomicOr(A.status, 1);
+    if (!finite(q.x) || !finite(q.y) || !finite(v.x) || !finite(v.y)) atomicOr(A.status, 1);
     A.y[i] = q;
     A.vel[i] = v;
 }
@@ -271,10 +288,11 @@ void launch_update(hts_ctx *c, double exag, double lr, double mom, double2 *g_ou
     A.seg_of = c->nseg > 1 ? c->seg_of : nullptr;
     A.seg_lr = c->seg_lr;
     A.seg_off = c->seg_off;
-    A.exag = exag;
-    A.lr = lr;
+    A.exag4 = 4.0 * exag;
+    A.lr = lr * (c->cfg.metric_pow == 2 ? 0.25 : 0.5);
     A.mom = mom;
     A.eps = c->cfg.eps;
+    A.lim2 = (1.0 - A.eps / 2.0) * (1.0 - A.eps / 2.0);
     A.metric_pow = c->cfg.metric_pow;
     A.use_gains = c->cfg.use_gains;
     A.do_step = do_step;
