@@ -430,115 +430,137 @@ __device__ __forceinline__ FX3 prefix_at(const EmitArgs &A, int p)
     return A.block_prefix && p < A.n ? fx3_add(A.block_prefix[p / kScanB], v) : v;
 }
 
-__global__ void emit_kernel(EmitArgs A)
+// The node of quadtree cell k (a binary internal node).
+__device__ __forceinline__ void emit_cell(const EmitArgs &A, int k)
 {
+    const int n = A.n;
+    int lo = A.lo_arr[k], hi = A.hi_arr[k];
+    int ell = quad_level(A.pref[k]);
+    int rank = __popc(A.mask[lo] & ((1u << ell) - 1u));  // shallower cells starting at lo
+    int pos = A.pre[lo] + rank;
+    int skip = A.pre[hi + 1];
+    const FX3 p1 = prefix_at(A, hi + 1), p0 = prefix_at(A, lo);
+    double cx, cy, beta;
+    if (A.nodes64 || A.ex.depth) {  // float64 walk / export: the oracle's correctly rounded steps
+        const int E = fx_exponent(*A.gmax, n);
+        const double sg = fx_to_double(p1.g - p0.g, E);
+        const double sux = fx_to_double(p1.x - p0.x, E);
+        const double suy = fx_to_double(p1.y - p0.y, E);
+        const double mx = __ddiv_rn(sux, sg);
+        const double my = __ddiv_rn(suy, sg);
+        const double sq = __dsqrt_rn(__dsub_rn(1.0, __dadd_rn(__dmul_rn(mx, mx), __dmul_rn(my, my))));
+        cx = __ddiv_rn(mx, __dadd_rn(1.0, sq));
+        cy = __ddiv_rn(my, __dadd_rn(1.0, sq));
+        beta = __dsub_rn(1.0, __dadd_rn(__dmul_rn(cx, cx), __dmul_rn(cy, cy)));
+    } else {
+        // float32 nodes: the sums stay scaled by 2^E (it cancels), and
+        // with m = S_u / S_g and R = sqrt(S_g^2 - |S_u|^2) = S_g sq,
+        //   y_cell = m / (1 + sq) = S_u / (S_g + R),
+        //   1 - |y_cell|^2 = 2 sq / (1 + sq) = 2 R / (S_g + R):
+        // one reciprocal instead of two
+        const double sg = fx_to_double_unscaled(p1.g - p0.g);
+        const double sux = fx_to_double_unscaled(p1.x - p0.x), suy = fx_to_double_unscaled(p1.y - p0.y);
+        const double R = sqrt(fmax(sg * sg - (sux * sux + suy * suy), 0.0));
+        const double rd = 1.0 / (sg + R);
+        cx = sux * rd;
+        cy = suy * rd;
+        beta = 2.0 * R * rd;
+    }
+    // 1 / beta: a float64 division for float64 nodes; float32 nodes store a
+    // float, taken as the float reciprocal of beta (off the float64 pipe)
+    const double il = A.nodes64 ? 1.0 / beta : 0.0;
+    const uint64_t key = A.keys[lo];
+    const int seg = (int)(key >> kSegShift);  // segment: its own root annulus
+    double lob = __longlong_as_double((long long)A.mm[2 * seg]);
+    double hib = __longlong_as_double((long long)A.mm[2 * seg + 1]);
+    const uint64_t kb = key & ((1ull << kSegShift) - 1);
+    uint64_t prefix = ell > 0 ? (kb >> (2 * (kLevels - ell))) : 0ull;
+    // float64 geometry for the float64 walk and for exports; float32 otherwise
+    const bool geo64 = A.nodes64 != nullptr || A.ex.depth != nullptr;
+    double rc = HUGE_VAL, thr = HUGE_VAL;
+    float thr32 = INFINITY;
+    if (ell > 0 && geo64) {
+        rc = cell_size(lob, hib, radial_index(prefix, ell), ell, A.rule);
+        if (A.theta > 0.0) {
+            double sh = sinh(rc / (2.0 * A.theta));
+            thr = 2.0 * sh * sh;
+        }
+        thr32 = (float)thr;
+    } else if (ell > 0 && A.theta > 0.0) {
+        thr32 = cell_threshold_f32(lob, hib, radial_index(prefix, ell), ell, A.rule, A.theta);
+    }
+    int count = hi - lo + 1;
+    bool bucket = ell == kLevels;
+    if (pos < 0 || pos >= A.capacity || skip <= pos || skip > A.capacity) {
+        atomicOr(A.status, 2);
+        return;
+    }
+    if (A.nodes32) {
+        NodeF nd;
+        float b32, unused;
+        split_f32(cx, nd.xh, nd.xl);
+        split_f32(cy, nd.yh, nd.yl);
+        split_f32(beta, b32, unused);  // (float)beta
+        nd.il = bucket ? __int_as_float(lo) : A.nodes64 ? (float)il : __frcp_rn(b32);
+        nd.thr = bucket ? -1.0f : thr32;
+        nd.count = bucket ? -count : count;
+        nd.skip = skip;
+        A.nodes32[pos] = nd;
+    }
+    if (A.nodes64) {
+        NodeD nd;
+        nd.x = cx;
+        nd.y = cy;
+        nd.il = il;
+        nd.thr = thr;
+        nd.count = bucket ? -count : count;
+        nd.skip = skip;
+        nd.pos = lo;
+        nd.pad = 0;
+        A.nodes64[pos] = nd;
+    }
+    if (A.ex.depth) {
+        int64_t first = -1;
+        if (bucket) {
+            first = A.idx[lo];
+            for (int p = lo + 1; p <= hi; ++p) first = min(first, (int64_t)A.idx[p]);
+        }
+        A.ex.depth[pos] = ell;
+        A.ex.prefix[pos] = prefix;
+        A.ex.count[pos] = count;
+        A.ex.first[pos] = first;
+        A.ex.ycell[2 * pos] = cx;
+        A.ex.ycell[2 * pos + 1] = cy;
+        A.ex.rcell[pos] = rc;
+    }
+}
+
+// The cells' float64 operations bound it (68% of that pipe), and only some of
+// the binary nodes are cells: a block first collects its cells, so that its
+// warps work on full ones (N = 1M: 123 us; 147 us with a lane per binary
+// node).  Then a lane per point writes the leaves.
+__global__ void __launch_bounds__(kBlock) emit_kernel(EmitArgs A)
+{
+    __shared__ int cells[kBlock], wcount[kBlock / 32];
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = A.n;
     if (k == 0 && A.nodes32) {  // empty slots after the last node: the float32 walk's overrun
         const int m = min(A.pre[n], A.capacity);
         for (int e = 0; e < kWalkOverrun; ++e) A.nodes32[m + e] = NodeF{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, m + e + 1};
     }
-    if (k < n - 1 && A.quad[k]) {
-        int lo = A.lo_arr[k], hi = A.hi_arr[k];
-        int ell = quad_level(A.pref[k]);
-        int rank = __popc(A.mask[lo] & ((1u << ell) - 1u));  // shallower cells starting at lo
-        int pos = A.pre[lo] + rank;
-        int skip = A.pre[hi + 1];
-        const FX3 p1 = prefix_at(A, hi + 1), p0 = prefix_at(A, lo);
-        double cx, cy, beta;
-        if (A.nodes64 || A.ex.depth) {  // float64 walk / export: the oracle's correctly rounded steps
-            const int E = fx_exponent(*A.gmax, n);
-            const double sg = fx_to_double(p1.g - p0.g, E);
-            const double sux = fx_to_double(p1.x - p0.x, E);
-            const double suy = fx_to_double(p1.y - p0.y, E);
-            const double mx = __ddiv_rn(sux, sg);
-            const double my = __ddiv_rn(suy, sg);
-            const double sq = __dsqrt_rn(__dsub_rn(1.0, __dadd_rn(__dmul_rn(mx, mx), __dmul_rn(my, my))));
-            cx = __ddiv_rn(mx, __dadd_rn(1.0, sq));
-            cy = __ddiv_rn(my, __dadd_rn(1.0, sq));
-            beta = __dsub_rn(1.0, __dadd_rn(__dmul_rn(cx, cx), __dmul_rn(cy, cy)));
-        } else {
-            // float32 nodes: the sums stay scaled by 2^E (it cancels), and
-            // with m = S_u / S_g and R = sqrt(S_g^2 - |S_u|^2) = S_g sq,
-            //   y_cell = m / (1 + sq) = S_u / (S_g + R),
-            //   1 - |y_cell|^2 = 2 sq / (1 + sq) = 2 R / (S_g + R):
-            // one reciprocal instead of two
-            const double sg = fx_to_double_unscaled(p1.g - p0.g);
-            const double sux = fx_to_double_unscaled(p1.x - p0.x), suy = fx_to_double_unscaled(p1.y - p0.y);
-            const double R = sqrt(fmax(sg * sg - (sux * sux + suy * suy), 0.0));
-            const double rd = 1.0 / (sg + R);
-            cx = sux * rd;
-            cy = suy * rd;
-            beta = 2.0 * R * rd;
-        }
-        // 1 / beta: a float64 division for float64 nodes; float32 nodes store a
-        // float, taken as the float reciprocal of beta (off the float64 pipe)
-        const double il = A.nodes64 ? 1.0 / beta : 0.0;
-        const uint64_t key = A.keys[lo];
-        const int seg = (int)(key >> kSegShift);  // segment: its own root annulus
-        double lob = __longlong_as_double((long long)A.mm[2 * seg]);
-        double hib = __longlong_as_double((long long)A.mm[2 * seg + 1]);
-        const uint64_t kb = key & ((1ull << kSegShift) - 1);
-        uint64_t prefix = ell > 0 ? (kb >> (2 * (kLevels - ell))) : 0ull;
-        // float64 geometry for the float64 walk and for exports; float32 otherwise
-        const bool geo64 = A.nodes64 != nullptr || A.ex.depth != nullptr;
-        double rc = HUGE_VAL, thr = HUGE_VAL;
-        float thr32 = INFINITY;
-        if (ell > 0 && geo64) {
-            rc = cell_size(lob, hib, radial_index(prefix, ell), ell, A.rule);
-            if (A.theta > 0.0) {
-                double sh = sinh(rc / (2.0 * A.theta));
-                thr = 2.0 * sh * sh;
-            }
-            thr32 = (float)thr;
-        } else if (ell > 0 && A.theta > 0.0) {
-            thr32 = cell_threshold_f32(lob, hib, radial_index(prefix, ell), ell, A.rule, A.theta);
-        }
-        int count = hi - lo + 1;
-        bool bucket = ell == kLevels;
-        if (pos < 0 || pos >= A.capacity || skip <= pos || skip > A.capacity) {
-            atomicOr(A.status, 2);
-            return;
-        }
-        if (A.nodes32) {
-            NodeF nd;
-            float b32, unused;
-            split_f32(cx, nd.xh, nd.xl);
-            split_f32(cy, nd.yh, nd.yl);
-            split_f32(beta, b32, unused);  // (float)beta
-            nd.il = bucket ? __int_as_float(lo) : A.nodes64 ? (float)il : __frcp_rn(b32);
-            nd.thr = bucket ? -1.0f : thr32;
-            nd.count = bucket ? -count : count;
-            nd.skip = skip;
-            A.nodes32[pos] = nd;
-        }
-        if (A.nodes64) {
-            NodeD nd;
-            nd.x = cx;
-            nd.y = cy;
-            nd.il = il;
-            nd.thr = thr;
-            nd.count = bucket ? -count : count;
-            nd.skip = skip;
-            nd.pos = lo;
-            nd.pad = 0;
-            A.nodes64[pos] = nd;
-        }
-        if (A.ex.depth) {
-            int64_t first = -1;
-            if (bucket) {
-                first = A.idx[lo];
-                for (int p = lo + 1; p <= hi; ++p) first = min(first, (int64_t)A.idx[p]);
-            }
-            A.ex.depth[pos] = ell;
-            A.ex.prefix[pos] = prefix;
-            A.ex.count[pos] = count;
-            A.ex.first[pos] = first;
-            A.ex.ycell[2 * pos] = cx;
-            A.ex.ycell[2 * pos + 1] = cy;
-            A.ex.rcell[pos] = rc;
-        }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool cell = k < n - 1 && A.quad[k];
+    const unsigned mine = __ballot_sync(0xffffffffu, cell);
+    if (lane == 0) wcount[w] = __popc(mine);
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int v = 0; v < kBlock / 32; ++v) {
+        before += v < w ? wcount[v] : 0;
+        total += wcount[v];
     }
+    if (cell) cells[before + __popc(mine & ((1u << lane) - 1u))] = k;
+    __syncthreads();
+    if ((int)threadIdx.x < total) emit_cell(A, cells[threadIdx.x]);
     if (k < n) {
         bool leaf = n == 1 || quad_level(A.pref[A.leaf_parent[k]]) < kLevels;
         int pos = A.pre[k] + A.cnt[k] - 1;
