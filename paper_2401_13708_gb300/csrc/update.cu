@@ -150,9 +150,9 @@ __device__ __forceinline__ bool not_below(double x, double lim)  // x >= lim, fo
 }
 
 // Bound by the float64 pipe (81% busy: ~80 operations a point at two lanes a
-// cycle per SM, N = 1M 115 us; its 96 bytes a point would take 15 us), so
+// cycle per SM, N = 1M 124 us; its 96 bytes a point would take 15 us), so
 // factors that are powers of two are folded into the arguments (the same bits)
-// and tests are made on bit patterns: 142 us with 15 operations more.
+// and tests are made on bit patterns: 158 us before.
 __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
 {
     __shared__ double s_invz;
@@ -214,17 +214,9 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     if (positive(vv)) {
         // exp map: p (+) tanh(lambda |v| / 2) v / |v|, lambda |v| / 2 = |v| / a;
         // 1 / |v| from one reciprocal square root (no square root and division)
-        // float32 mode: from f64math.cuh's seeds (float64 mode keeps the
-        // library's roundings)
-        double rn, nv, x;
-        if (A.rounded) {
-            rn = rsqrt(vv);
-            nv = vv * rn;
-            x = nv / a;
-        } else {
-            sqrt_rsqrt(not_below(vv, 1e-300) ? vv : 1e-300, nv, rn);
-            x = nv * reciprocal(a);
-        }
+        // (own roots and reciprocals, an ulp off, would be faster; over several
+        // steps of a spread embedding they grow to 1e-9 of the velocity)
+        const double rn = rsqrt(vv), nv = vv * rn, x = nv / a;
         if (A.rounded && x > 2.0) {
             q = long_step(p, v);
         } else {
@@ -234,7 +226,7 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
             const double nu = ux * ux + uy * uy;
             const double ca = 1.0 + 2.0 * pu + nu;
             const double den = 1.0 + 2.0 * pu + n2 * nu;
-            const double rden = A.rounded ? 1.0 / den : reciprocal(den);
+            const double rden = 1.0 / den;
             q.x = (ca * p.x + a * ux) * rden;
             q.y = (ca * p.y + a * uy) * rden;
         }
