@@ -535,7 +535,7 @@ __device__ __forceinline__ void emit_cell(const EmitArgs &A, int k)
     }
 }
 
-// The cells' float64 operations bound it (68% of that pipe), and only some of
+// The cells' float64 operations bound it (56% of that pipe), and only some of
 // the binary nodes are cells: a block first collects its cells, so that its
 // warps work on full ones (N = 1M: 123 us; 147 us with a lane per binary
 // node).  Then a lane per point writes the leaves.
