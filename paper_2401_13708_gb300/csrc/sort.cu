@@ -374,27 +374,32 @@ namespace {
 // finds every key's place among all tiles the same way, the first steps of
 // each search in a sample of every 32nd key.  Equal keys stay in index order:
 // runs and tiles hold consecutive indices, so an earlier one's equal keys come
-// before and a later one's after.  (A bitonic sort of a
+// before and a later one's after.  The tail of the last tile is filled with
+// 2^64 - 1, which a point can have as its key too (segment 63, outermost, angle
+// just below a full turn): it is told from the points by its place alone, after
+// all of them, where the same counting leaves it.  (A bitonic sort of a
 // 2,048-key tile: 22 us.)
 constexpr int kRun = 64, kRun2 = 512, kSample = 32;
 template <int kTile> constexpr int kTileThreads = kTile < 1024 ? kTile : 1024;
 
-// Keys of a sorted run (kLen, a power of two) that are below lim.
+// Keys of a sorted run (kLen, a power of two) that go before `key`: those below
+// it and, in a run of earlier indices, those equal to it (below key + 1, or all
+// of them where that wraps).
 template <int kLen>
-__device__ __forceinline__ int count_below(const uint64_t *run, uint64_t lim)
+__device__ __forceinline__ int count_before(const uint64_t *run, uint64_t key, bool earlier)
 {
+    const uint64_t lim = key + (earlier ? 1ull : 0ull);
     int c = 0;
 #pragma unroll
     for (int s = kLen >> 1; s > 0; s >>= 1)
         if (run[c + s - 1] < lim) c += s;
-    return c + (run[c] < lim ? 1 : 0);
+    c += run[c] < lim ? 1 : 0;
+    return earlier && key == ~0ull ? kLen : c;
 }
 
-// Merges groups of kLen-key runs (kGroup keys each) of `k` into `ko`.  Padding
-// keys (2^64 - 1, the tail of the tile) are larger than every key and already
-// in the last places of their group: they stay where they are.
+// Merges groups of kLen-key runs (kGroup keys each) of `k` into `ko`.
 template <int kTile, int kLen, int kGroup>
-__device__ __forceinline__ void merge_padded(const uint64_t *k, const uint16_t *v, uint64_t *ko, uint16_t *vo)
+__device__ __forceinline__ void merge_runs(const uint64_t *k, const uint16_t *v, uint64_t *ko, uint16_t *vo)
 {
 #pragma unroll
     for (int q = 0; q < kTile / kTileThreads<kTile>; ++q) {
@@ -404,10 +409,9 @@ __device__ __forceinline__ void merge_padded(const uint64_t *k, const uint16_t *
         int pos = e & (kLen - 1);
 #pragma unroll
         for (int r = 0; r < kGroup / kLen; ++r) {
-            const int c = count_below<kLen>(k + group + r * kLen, key + (r < own ? 1ull : 0ull));
+            const int c = count_before<kLen>(k + group + r * kLen, key, r < own);
             pos += r == own ? 0 : c;
         }
-        if (key == ~0ull) pos = e & (kGroup - 1);
         ko[group + pos] = key;
         vo[group + pos] = v[e];
     }
@@ -426,7 +430,7 @@ __global__ void __launch_bounds__(kTileThreads<kTile>) tile_sort_kernel(const ui
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
         const int e = threadIdx.x + q * kTileThreads<kTile>;
-        key[q] = base + e < n ? kin[base + e] : ~0ull;  // (padding: after every key)
+        key[q] = base + e < n ? kin[base + e] : ~0ull;
         ka[e] = key[q];
     }
     __syncthreads();
@@ -435,23 +439,22 @@ __global__ void __launch_bounds__(kTileThreads<kTile>) tile_sort_kernel(const ui
         const int e = threadIdx.x + q * kTileThreads<kTile>;
         const uint64_t *run = ka + (e & ~(kRun - 1));
         const int half = e & 32;
-        const bool pad = key[q] == ~0ull;
-        const uint64_t next = key[q] + (pad ? 0ull : 1ull), other = half ? next : key[q];
+        const uint64_t next = key[q] + 1ull, other = half ? next : key[q];
         int rank = 0;
 #pragma unroll 8
         for (int j = 0; j < 32; ++j) {
             rank += run[(half ^ 32) + j] < other ? 1 : 0;
             rank += run[half + j] < (j < lane ? next : key[q]) ? 1 : 0;
         }
-        if (pad) rank = e & (kRun - 1);  // (a run's padding is its tail already)
+        if (key[q] == ~0ull) rank += e & (kRun - 1);  // (`next` wrapped: all the earlier ones)
         kb[(e & ~(kRun - 1)) + rank] = key[q];
         vb[(e & ~(kRun - 1)) + rank] = (uint16_t)e;
     }
     __syncthreads();
-    merge_padded<kTile, kRun, kRun2>(kb, vb, ka, va);
+    merge_runs<kTile, kRun, kRun2>(kb, vb, ka, va);
     __syncthreads();
     if (kTile > kRun2) {
-        merge_padded<kTile, kRun2, kTile>(ka, va, kb, vb);
+        merge_runs<kTile, kRun2, kTile>(ka, va, kb, vb);
         __syncthreads();
     }
     const uint64_t *ks = kTile > kRun2 ? kb : ka;
@@ -490,7 +493,7 @@ __global__ void __launch_bounds__(1024) rank_scatter_kernel(const uint64_t *__re
             const int t = t0 + q;
             at[q] = n;
             if (t < tiles && t != own) {
-                const int c = count_below<kPerTile>(sort_shared + t * kPerTile, key + (t < own ? 1ull : 0ull));
+                const int c = count_before<kPerTile>(sort_shared + t * kPerTile, key, t < own);
                 pos += c * kSample;
                 if (c < kPerTile) at[q] = t * kTile + c * kSample;
             }
@@ -500,6 +503,7 @@ __global__ void __launch_bounds__(1024) rank_scatter_kernel(const uint64_t *__re
 #pragma unroll
             for (int q = 0; q < kAtOnce; ++q) {  // (fewer than kSample smaller keys in the group)
                 const int p = at[q] + s - 1;
+                // (key + 1 wraps only where every key of the tile goes before: at[q] == n)
                 if (p < n && __ldg(kin + p) < key + (t0 + q < own ? 1ull : 0ull)) {
                     at[q] += s;
                     pos += s;
