@@ -1192,11 +1192,12 @@ __global__ void __launch_bounds__(kSumBlockD) sum_f64_kernel(int n, const NodeF 
     const int shares = kWarps * (int)gridDim.y, share = (int)blockIdx.y * kWarps + w;
     LaneD L;
     load_lane(L, chunk, lane, n, spts, leaf);
-    if (lv.direct[chunk]) {  // (the same for the whole block)
-        if (share > 0) return;
-        walk_f64_chunk<GF, false, false, false>(L, n, lane, nodes, nodes64, n_nodes, spts, nullptr, SegView{}, nullptr,
-                                                0, S.tile);
-        store_lane(L, 0, n, idx, frep, zi, gridDim.y > 1 ? sp.part : nullptr);
+    if (lv.direct[chunk]) {  // (the same for all the chunk's blocks)
+        if (w > 0) return;
+        if (blockIdx.y == 0)  // (the other blocks' sums are zero: every block's are added)
+            walk_f64_chunk<GF, false, false, false>(L, n, lane, nodes, nodes64, n_nodes, spts, nullptr, SegView{},
+                                                    nullptr, 0, S.tile);
+        store_lane(L, blockIdx.y, n, idx, frep, zi, gridDim.y > 1 ? sp.part : nullptr);
         return;
     }
     // batches of up to 32 interactions from consecutive pages, dealt to the
