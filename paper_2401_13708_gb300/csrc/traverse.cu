@@ -149,8 +149,11 @@ struct NodesF {  // cell test, points and skip index
 // Interaction lists between list_f32_kernel and sum_f32_kernel: pages of up
 // to 32 interactions (the node and the lanes of the chunk that take it).  The
 // first page of every (chunk, unit) has a fixed place; further ones come from
-// pools (chunk mod kListPools, so that the atomic counters are spread).  A
-// chunk whose pool runs out is flagged and walked directly by sum_f32_kernel.
+// pools (chunk mod kListPools, so that the atomic counters are spread).  Where
+// a pool runs out, float32 chunks that found it empty are flagged and walked
+// directly by sum_f32_kernel (the same sums).  Direct float64 sums differ in
+// their last bits, and which chunk finds the pool empty depends on timing: there
+// all chunks of the pool are walked directly (ran_out).
 constexpr int kPage = 32;
 constexpr int kListPools = 256;
 
@@ -158,10 +161,13 @@ struct ListView {
     uint2 *entries;    // [page][kPage]: node, lane mask
     int2 *head;        // per page: interactions held, next page (-1: none)
     int *taken;        // per pool: pages taken
-    int *direct;       // per chunk: its pool ran out
+    int *direct;       // per chunk: it found its pool empty
     int units;         // first pages per chunk
     int chunks;
     int per_pool;      // further pages per pool
+    // more pages were asked for than the pool has: the same in every run (a
+    // warp asks until it is done or is refused)
+    __device__ bool ran_out(int chunk) const { return taken[chunk & (kListPools - 1)] > per_pool; }
 };
 
 // Per-lane state of the float32 walk: the query point (sorted position p),
@@ -1192,7 +1198,7 @@ __global__ void __launch_bounds__(kSumBlockD) sum_f64_kernel(int n, const NodeF 
     const int shares = kWarps * (int)gridDim.y, share = (int)blockIdx.y * kWarps + w;
     LaneD L;
     load_lane(L, chunk, lane, n, spts, leaf);
-    if (lv.direct[chunk]) {  // (the same for all the chunk's blocks)
+    if (lv.ran_out(chunk)) {  // (the same for all the chunk's blocks)
         if (w > 0) return;
         if (blockIdx.y == 0)  // (the other blocks' sums are zero: every block's are added)
             walk_f64_chunk<GF, false, false, false>(L, n, lane, nodes, nodes64, n_nodes, spts, nullptr, SegView{},

@@ -1,7 +1,7 @@
 """Interaction lists that do not fit their pages, in float64: a tight cluster with
 outliers at nested distances is cut into a few units only (a cut stops at eight
 ancestors), so that at theta = 0.005 the pools of two chunks run out (9,728
-points: 48 of the 256).  Such chunks are walked directly by one of the two
+points: 48 of the 256).  Their chunks are walked directly by one of the two
 blocks that sum a chunk; the other adds nothing."""
 import numpy as np
 import pytest
@@ -41,3 +41,16 @@ def test_overflow_after_a_call_that_left_sums(form):
         g2, z2 = t.grad(THETA)
     assert abs(z - z2) <= TOL * abs(z2)
     assert np.linalg.norm(g - g2) <= TOL * np.linalg.norm(g2)
+
+
+def test_overflow_gives_the_same_bits_again():
+    """131,071 points at theta = 0.2: pools of 16 chunks run out, and which chunk
+    finds its pool empty depends on timing."""
+    n = 131071
+    with HyperbolicTSNE(precision="fp64") as t:
+        t.set_P(np.zeros(n + 1, np.int64), np.zeros(0, np.int32), np.zeros(0, np.float64))
+        t.set_Y(inputs.spread_embedding(np.arange(n) % 20, 3, rho_hi=6.0))
+        g, z = t.grad(0.2)
+        for _ in range(5):
+            h, y = t.grad(0.2)
+            assert np.array_equal(g, h) and z == y
