@@ -1671,7 +1671,9 @@ void launch_walk(hts_ctx *c)
     const bool fp64 = c->cfg.precision == HTS_FP64;
     const int depth = seg ? 0 : walk_split_depth(n, c->walk_split, fp64);
     // (float64: a depth that was asked for is the cut of the direct walk)
-    const bool list = !seg && (!fp64 || c->walk_split < 0) && !cnt && list_units(n, fp64) > 0;
+    // (the counting walk is direct: the same bits in float32; in float64, where they
+    // would differ, it runs before the listed one and only counts)
+    const bool list = !seg && (fp64 ? c->walk_split < 0 : !cnt) && list_units(n, fp64) > 0;
     const int blocks64 = fp64 && list ? f64_sum_blocks(c) : 1;
     const bool split = fp64 && list ? blocks64 > 1 : depth > 0;
     SplitView sp{nullptr, nullptr};
@@ -1723,6 +1725,17 @@ void launch_walk(hts_ctx *c)
         const dim3 lgrid((unsigned)((warps * 32 + kListBlock - 1) / kListBlock), (unsigned)lv.units);
         c->launches += 1;
         if (fp64) {
+            if (cnt) {
+                if (c->cfg.grad_form == HTS_EXACT_KL)
+                    walk_f64_kernel<0, true, false, false><<<dim3(grid.x), block, 0, c->stream>>>(
+                        n, c->nodes32, c->nodes64, c->n_nodes, c->spts64, c->cnt, c->idx, c->frep, c->zi, c->counters, sv,
+                        SplitView{nullptr, nullptr}, bo);
+                else
+                    walk_f64_kernel<1, true, false, false><<<dim3(grid.x), block, 0, c->stream>>>(
+                        n, c->nodes32, c->nodes64, c->n_nodes, c->spts64, c->cnt, c->idx, c->frep, c->zi, c->counters, sv,
+                        SplitView{nullptr, nullptr}, bo);
+                c->launches += 1;
+            }
             list_f64_kernel<<<lgrid, kListBlock, 0, c->stream>>>(n, c->nodes32, c->nodes64, c->spts64, c->cnt, sp.cut, lv);
             const dim3 sgrid((unsigned)warps, (unsigned)blocks64);
             if (c->cfg.grad_form == HTS_EXACT_KL)
