@@ -1651,13 +1651,15 @@ int walk_split_depth(int64_t n, int want, bool fp64)
     return d;
 }
 
-// Blocks per chunk that sum a listed float64 walk: four blocks per SM while
-// there are fewer chunks than SMs (N = 2,000, two / four / six per SM: 124 /
-// 108 / 132 us).
-static int f64_sum_blocks(const hts_ctx *c)
+// Blocks per chunk that sum a listed float64 walk: four blocks on each of 152
+// SMs while there are fewer chunks than SMs (N = 2,000, two / four / six per SM:
+// 124 / 108 / 132 us).  The number decides the order of the sums, so it follows
+// from the size alone, not from the SMs of the device at hand.
+static int f64_sum_blocks(int64_t n)
 {
-    const int64_t chunks = std::max<int64_t>((c->n + 31) / 32, 1);
-    return (int)std::max<int64_t>(1, std::min<int64_t>(4 * c->sm_count / chunks, std::min(16, walk_split_capacity(c->n))));
+    constexpr int64_t kTargetBlocks = 4 * 152;
+    const int64_t chunks = std::max<int64_t>((n + 31) / 32, 1);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kTargetBlocks / chunks, std::min(16, walk_split_capacity(n))));
 }
 
 void launch_walk(hts_ctx *c)
@@ -1674,7 +1676,7 @@ void launch_walk(hts_ctx *c)
     // (the counting walk is direct: the same bits in float32; in float64, where they
     // would differ, it runs before the listed one and only counts)
     const bool list = !seg && (fp64 ? c->walk_split < 0 : !cnt) && list_units(n, fp64) > 0;
-    const int blocks64 = fp64 && list ? f64_sum_blocks(c) : 1;
+    const int blocks64 = fp64 && list ? f64_sum_blocks(n) : 1;
     const bool split = fp64 && list ? blocks64 > 1 : depth > 0;
     SplitView sp{nullptr, nullptr};
     const AnnulusView an{c->minmax, seg ? c->keys : nullptr, c->cfg.split_rule, n - 1};
