@@ -287,13 +287,15 @@ HTS_API int hts_set_graphs(hts_ctx *ctx, int enable);
  * stream with CUDA events, keeps the fastest and writes the choice to
  * tuning[2] = {walk threads per block, attraction lanes per row} (may be
  * NULL); for a small problem it also picks the split walk's cut depth
- * (hts_get_walk_split).  A smaller walk block is kept only if it is 3% faster
- * than the larger ones.  It changes no result of the walk (the work split per warp does not
- * depend on the block size); lanes per row change only the float32 summation
- * order inside a row.  hts_set_tuning sets them directly (0 keeps a value),
- * hts_get_tuning reads them.  Defaults: {256, 8}.  Errors: HTS_ENOTSET,
- * HTS_EINVAL (theta outside [0, 1], reps outside [1, 1000], a value not in
- * the lists), HTS_ECUDA. */
+ * (hts_get_walk_split), in float64 with the default (depth -1) among the
+ * candidates, which is kept unless a depth is 3% faster.  A smaller walk block
+ * is kept only if it is 3% faster than the larger ones, and none is timed where
+ * the walk has no block size (hts_set_walk_split).  The block size changes no
+ * result; another depth changes the order of the walk's sums, and lanes per row
+ * change the float32 summation order inside a row.  hts_set_tuning sets them
+ * directly (0 keeps a value), hts_get_tuning reads them.  Defaults: {256, 8}.
+ * Errors: HTS_ENOTSET, HTS_EINVAL (theta outside [0, 1], reps outside
+ * [1, 1000], a value not in the lists), HTS_ECUDA. */
 HTS_API int hts_autotune(hts_ctx *ctx, double theta, int reps, int *tuning);
 
 /* Split walk for small problems (one embedding; no counterpart in the
@@ -305,11 +307,19 @@ HTS_API int hts_autotune(hts_ctx *ctx, double theta, int reps, int *tuning);
  * exactly the interactions of its own walk (the partial sums are added in a
  * fixed order).  depth = -1 (default) picks the shallowest cut that gives
  * about 2048 warps, within a partial-sum buffer of
- * min(64 n, 2^22) entries for n <= 524288 (no split above).  Errors: HTS_EINVAL (depth < -1 or > 3). */
+ * min(64 n, 2^22) entries for n <= 524288 (no split above).
+ * Float32 walks of up to 32,768 points list their interactions first and sum
+ * them in the order of the walk, subtree by subtree of the cut.  Float64 walks
+ * of up to 262,144 points do so too at depth = -1 only, and share a point's
+ * interactions evenly among lanes: there the cut plays no part in the sums, and
+ * depth >= 0 asks for the walk that adds as it goes, cut at that depth (the
+ * same interactions in another order: the last bits differ).  Errors:
+ * HTS_EINVAL (depth < -1 or > 3). */
 HTS_API int hts_set_walk_split(hts_ctx *ctx, int depth);
 /* The cut depth in use (the automatic choice resolved; 0 with segments).
  * hts_autotune also times every depth the buffer allows on the current
- * problem and keeps the fastest.  Errors: HTS_EINVAL. */
+ * problem and keeps the fastest (float64: unless depth = -1 is as fast).
+ * Errors: HTS_EINVAL. */
 HTS_API int hts_get_walk_split(const hts_ctx *ctx, int *depth);
 HTS_API int hts_set_tuning(hts_ctx *ctx, int walk_block, int attract_lanes);
 HTS_API int hts_get_tuning(const hts_ctx *ctx, int *tuning);

@@ -1206,36 +1206,57 @@ int hts_autotune(hts_ctx *c, double theta, int reps, int *tuning)
             // tuning state (balance of the cost-ordered launches) tends to turn
             // into a loss as the embedding spreads, where larger blocks share
             // node data in L1 across more warps (N = 1M over the protocol: 128
-            // and 256 threads 3-8% ahead of 64, though 64 can win at Y0)
-            const int cand[4] = {256, 128, 64, 32};
-            float best = INFINITY;
-            int pick = c->walk_block;
-            for (int wb : cand) {
-                c->walk_block = wb;
-                float ms = 0.f;
-                if ((r = time_it([&] { launch_walk(c); }, &ms))) return r;
-                if (ms < 0.97f * best) {
-                    best = ms;
-                    pick = wb;
+            // and 256 threads 3-8% ahead of 64, though 64 can win at Y0).  A
+            // listed walk has no block size to tune.
+            auto tune_block = [&]() -> int {
+                if (walk_lists(c)) return HTS_OK;
+                const int cand[4] = {256, 128, 64, 32};
+                float best = INFINITY;
+                int pick = c->walk_block;
+                for (int wb : cand) {
+                    c->walk_block = wb;
+                    float ms = 0.f;
+                    int e = time_it([&] { launch_walk(c); }, &ms);
+                    if (e) return e;
+                    if (ms < 0.97f * best) {
+                        best = ms;
+                        pick = wb;
+                    }
                 }
-            }
-            c->walk_block = pick;
-            // warps per chunk: the cut depth of the split walk (small problems)
-            const int dmax = walk_split_depth(c->n, kMaxSplitCut, c->cfg.precision == HTS_FP64);
+                c->walk_block = pick;
+                return HTS_OK;
+            };
+            // warps per chunk: the cut depth of the split walk (small problems).
+            // In float64 a depth stands for the direct walk and -1 for the
+            // listed one, which is kept unless a depth is 3% faster (N = 2,000:
+            // 0.32 ms listed, 0.68 direct at its best depth; 70,000: 9.0 and 9.6;
+            // 131,071 at theta = 1: 6.5 and 6.4); the block is then that of the
+            // form that is kept.
+            const bool fp64 = c->cfg.precision == HTS_FP64;
+            struct Uncounted {  // (a counted listed walk is two walks)
+                hts_ctx *c;
+                int keep;
+                ~Uncounted() { c->counters_on = keep; }
+            } uncounted{c, c->counters_on};
+            if (fp64) c->counters_on = 0;
+            const int dmax = walk_split_depth(c->n, kMaxSplitCut, fp64);
+            if (!fp64 && (r = tune_block())) return r;
             if (c->nseg == 1 && dmax > 0) {
                 float bestd = INFINITY;
                 int pickd = 0;
-                for (int d = 0; d <= dmax; ++d) {
+                c->walk_split = -1;
+                for (int d = fp64 && walk_lists(c) ? -1 : 0; d <= dmax; ++d) {
                     c->walk_split = d;
                     float ms = 0.f;
                     if ((r = time_it([&] { launch_walk(c); }, &ms))) return r;
-                    if (ms < bestd) {
+                    if (ms < (pickd < 0 ? 0.97f : 1.0f) * bestd) {
                         bestd = ms;
                         pickd = d;
                     }
                 }
                 c->walk_split = pickd;
             }
+            if (fp64 && (r = tune_block())) return r;
         }
         if (c->nnz > 0 && c->cfg.precision == HTS_FP32_MIXED) {
             const int cand[4] = {4, 8, 16, 32};

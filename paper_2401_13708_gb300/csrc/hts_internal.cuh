@@ -245,6 +245,7 @@ int exact_split(int64_t n);
 int walk_split_capacity(int64_t n);
 int walk_split_depth(int64_t n, int want, bool fp64);
 size_t walk_split_frontier_bytes();
+bool walk_lists(const hts_ctx *c);
 // interaction lists: pages for n points, bytes of a page, counters and flags
 int64_t list_pages(int64_t n, bool fp64);
 size_t list_page_bytes();

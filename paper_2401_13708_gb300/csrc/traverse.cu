@@ -1662,6 +1662,15 @@ static int f64_sum_blocks(int64_t n)
     return (int)std::max<int64_t>(1, std::min<int64_t>(kTargetBlocks / chunks, std::min(16, walk_split_capacity(n))));
 }
 
+// Whether launch_walk lists the interactions first (float64: a depth that was
+// asked for is the cut of the direct walk; float32: the counting walk is direct,
+// with the same bits).
+bool walk_lists(const hts_ctx *c)
+{
+    const bool fp64 = c->cfg.precision == HTS_FP64;
+    return c->nseg == 1 && (fp64 ? c->walk_split < 0 : !c->counters_on) && list_units(c->n, fp64) > 0;
+}
+
 void launch_walk(hts_ctx *c)
 {
     const int n = (int)c->n;
@@ -1672,10 +1681,7 @@ void launch_walk(hts_ctx *c)
     const SegView sv{c->keys, c->seg_off, c->pre};
     const bool fp64 = c->cfg.precision == HTS_FP64;
     const int depth = seg ? 0 : walk_split_depth(n, c->walk_split, fp64);
-    // (float64: a depth that was asked for is the cut of the direct walk)
-    // (the counting walk is direct: the same bits in float32; in float64, where they
-    // would differ, it runs before the listed one and only counts)
-    const bool list = !seg && (fp64 ? c->walk_split < 0 : !cnt) && list_units(n, fp64) > 0;
+    const bool list = walk_lists(c);
     const int blocks64 = fp64 && list ? f64_sum_blocks(n) : 1;
     const bool split = fp64 && list ? blocks64 > 1 : depth > 0;
     SplitView sp{nullptr, nullptr};
@@ -1727,7 +1733,7 @@ void launch_walk(hts_ctx *c)
         const dim3 lgrid((unsigned)((warps * 32 + kListBlock - 1) / kListBlock), (unsigned)lv.units);
         c->launches += 1;
         if (fp64) {
-            if (cnt) {
+            if (cnt) {  // (the direct walk's float64 sums differ in their last bits: it only counts)
                 if (c->cfg.grad_form == HTS_EXACT_KL)
                     walk_f64_kernel<0, true, false, false><<<dim3(grid.x), block, 0, c->stream>>>(
                         n, c->nodes32, c->nodes64, c->n_nodes, c->spts64, c->cnt, c->idx, c->frep, c->zi, c->counters, sv,
