@@ -96,6 +96,24 @@ __global__ void empty_nodes_kernel(int64_t slots, NodeF *nodes)
     if (k < slots) nodes[k] = NodeF{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, (int)(k + 1)};
 }
 
+void drop_lists(hts_ctx *c)
+{
+    dfree(&c->list_entries);
+    c->lists_refused = 0;
+}
+
+// Float32 node slots: one never written by a tree build reads as an empty bucket
+// (count 0), which the walk steps over (its skip is its index + 1).
+int alloc_nodes32(hts_ctx *c, size_t N)
+{
+    const int64_t slots = (int64_t)(2 * N + kWalkOverrun);
+    int r = dalloc(c, &c->nodes32, (size_t)slots);
+    if (r) return r;
+    empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256>>>(slots, c->nodes32);
+    if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return HTS_ECUDA;
+    return HTS_OK;
+}
+
 int ensure_points(hts_ctx *c, int64_t n)
 {
     if (n == c->cap_n && (c->pts32 || c->pts64)) return HTS_OK;
@@ -115,19 +133,14 @@ int ensure_points(hts_ctx *c, int64_t n)
         AL(c->pts32, N);
         AL(c->apts32, N);
         AL(c->spts32, N);
+        if ((r = alloc_nodes32(c, N))) return r;
     } else {
         AL(c->pts64, N);
         AL(c->spts64, N);
         AL(c->nodes64, 2 * N);
+        dfree(&c->nodes32);
     }
-    AL(c->nodes32, 2 * N + kWalkOverrun);  // (in float64 mode they decide the criterion)
-    // a node slot never written by a tree build reads as an empty bucket
-    // (count 0), which the walk steps over (its skip is its index + 1)
-    if (c->nodes32) {
-        const int64_t slots = (int64_t)(2 * N + kWalkOverrun);
-        empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256>>>(slots, c->nodes32);
-        if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return HTS_ECUDA;
-    }
+    drop_lists(c);  // (and float64 mode's float32 nodes: ensure_nodes)
     if (c->nodes64 && cudaMemset(c->nodes64, 0, sizeof(NodeD) * 2 * N) != cudaSuccess) return HTS_ECUDA;
     AL(c->keys, N);
     AL(c->keys_alt, N);
@@ -173,16 +186,44 @@ int ensure_points(hts_ctx *c, int64_t n)
         c->split_part = part;
         c->split_frontier = fr;
     }
-    {
-        const size_t pages = (size_t)list_pages((int64_t)N, c->cfg.precision == HTS_FP64);
-        AL(c->list_entries, pages * (list_page_bytes() / sizeof(uint2)));
-        AL(c->list_head, pages);
-        AL(c->list_flags, (size_t)list_flags((int64_t)N));
-    }
 #undef AL
     c->n_nodes = c->pre + n;
     c->cap_n = n;
     return HTS_OK;
+}
+
+// What a tree walk needs beyond ensure_points' buffers is taken by the first call
+// that walks (theta = 0 never does, segments never list): float64 mode's float32
+// nodes, which decide its criterion (64 bytes a point), and the interaction
+// lists (up to 175 MB at 32,768 points in float32, 570 MB at 262,144 in
+// float64).  run_gradient asks for the lists once the tree build is queued, so
+// that their allocation runs beside it (N = 20,011: the first gradient takes 48 us
+// more, hts_set_Y before it 50 us less than with the lists taken there).  Lists that do not fit
+// are left out until the size changes: the walk is then the direct one.
+int ensure_nodes(hts_ctx *c)
+{
+    if (c->nodes32 || c->n == 0) return HTS_OK;
+    c->layout_version += 1;
+    return alloc_nodes32(c, (size_t)c->n);
+}
+
+void ensure_lists(hts_ctx *c)
+{
+    if (c->list_entries || c->lists_refused || !walk_wants_lists(c)) return;
+    // one block: entries, heads, flags
+    const size_t pages = (size_t)list_pages(c->n, c->cfg.precision == HTS_FP64);
+    const size_t entries = pages * (list_page_bytes() / sizeof(uint2));
+    const size_t flags = ((size_t)list_flags(c->n) + 1) / 2;
+    static_assert(sizeof(int2) == sizeof(uint2) && 2 * sizeof(int) == sizeof(uint2), "units of the block");
+    if (dalloc(c, &c->list_entries, entries + pages + flags) == HTS_OK) {
+        c->list_head = reinterpret_cast<int2 *>(c->list_entries + entries);
+        c->list_flags = reinterpret_cast<int *>(c->list_entries + entries + pages);
+    } else {
+        cudaGetLastError();
+        c->err.clear();
+        c->lists_refused = 1;
+    }
+    c->layout_version += 1;
 }
 
 int read_status(hts_ctx *c, int *out)
@@ -257,6 +298,7 @@ int run_gradient(hts_ctx *c, double theta, cudaEvent_t *ev = nullptr)
         launch_exact(c);
         LAUNCHED("exact");
     } else {
+        if ((r = ensure_nodes(c))) return r;
         if (attract && fork_at == 0 && (r = fork_attract())) return r;
         launch_make_keys(c);
         LAUNCHED("make_keys");
@@ -270,6 +312,7 @@ int run_gradient(hts_ctx *c, double theta, cudaEvent_t *ev = nullptr)
         LAUNCHED("build_tree");
         MARK(3);
         if (attract && fork_at == 3 && (r = fork_attract())) return r;
+        ensure_lists(c);
         launch_walk(c);
         LAUNCHED("walk");
     }
@@ -339,6 +382,11 @@ void drop_graph(hts_ctx *c)
 // stream, unless the cached graph already matches the arguments and layout.
 int capture_iteration(hts_ctx *c, double theta, double exag, double lr, double mom)
 {
+    if (theta > 0.0) {  // (nothing is allocated in a capture)
+        const int r = ensure_nodes(c);
+        if (r) return r;
+        ensure_lists(c);
+    }
     const double key[5] = {theta, exag, lr, mom, (double)c->layout_version};
     if (c->gexec && memcmp(key, c->gkey, sizeof(key)) == 0) return HTS_OK;
     drop_graph(c);
@@ -526,7 +574,7 @@ void hts_destroy(hts_ctx *c)
     dfree(&c->bn_lo); dfree(&c->bn_hi); dfree(&c->bn_pref); dfree(&c->bn_flag); dfree(&c->bn_quad);
     dfree(&c->bn_sum); dfree(&c->cnt); dfree(&c->pre); dfree(&c->nodes32); dfree(&c->apts32); dfree(&c->walk_cost); dfree(&c->walk_order); dfree(&c->nodes64);
     dfree(&c->sort_scratch); dfree(&c->scan_tmp); dfree(&c->exact_part);
-    dfree(&c->list_entries); dfree(&c->list_head); dfree(&c->list_flags);
+    dfree(&c->list_entries);
     if (c->split_part) cudaFree(c->split_part);
     if (c->split_frontier) cudaFree(c->split_frontier); dfree(&c->red_tmp); dfree(&c->minmax);
     dfree(&c->dscal); dfree(&c->status); dfree(&c->counters); dfree(&c->xsq);
@@ -1184,6 +1232,11 @@ int hts_autotune(hts_ctx *c, double theta, int reps, int *tuning)
     if (c->n > 0) {
         CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
         if ((r = ensure_events(c, 1))) return r;
+        const int keep_split = c->walk_split;
+        c->walk_split = -1;  // (with the lists: the depths are timed below)
+        if (theta > 0.0) ensure_lists(c);
+        c->walk_split = keep_split;
+        if (theta > 0.0 && (r = ensure_nodes(c))) return r;
         cudaEvent_t a = c->events[0], b = c->events[1];
         launch_prep_points(c);
         LAUNCHED("prep_points");

@@ -193,7 +193,8 @@ struct hts_ctx {
     unsigned *walk_cost = nullptr;   // per walk block: cycles of the last walk (launch-order input)
     int *walk_order = nullptr;       // [0] grid size, then the launch order of the walk's blocks
     void *split_frontier = nullptr;  // cuts of the tree (CutTables)
-    uint2 *list_entries = nullptr;   // interaction lists of the float32 walk: pages of 32 entries,
+    int lists_refused = 0;           // the interaction lists did not fit (ensure_lists)
+    uint2 *list_entries = nullptr;   // interaction lists, from the first walk that wants them (one block): pages of 32 entries,
     int2 *list_head = nullptr;       //   entries and next page of each page,
     int *list_flags = nullptr;       //   pages taken per pool, then a flag per chunk
     void *split_part = nullptr;      // partial sums of the split walk
@@ -245,6 +246,7 @@ int exact_split(int64_t n);
 int walk_split_capacity(int64_t n);
 int walk_split_depth(int64_t n, int want, bool fp64);
 size_t walk_split_frontier_bytes();
+bool walk_wants_lists(const hts_ctx *c);
 bool walk_lists(const hts_ctx *c);
 // interaction lists: pages for n points, bytes of a page, counters and flags
 int64_t list_pages(int64_t n, bool fp64);

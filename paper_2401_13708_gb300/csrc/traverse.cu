@@ -1662,14 +1662,16 @@ static int f64_sum_blocks(int64_t n)
     return (int)std::max<int64_t>(1, std::min<int64_t>(kTargetBlocks / chunks, std::min(16, walk_split_capacity(n))));
 }
 
-// Whether launch_walk lists the interactions first (float64: a depth that was
-// asked for is the cut of the direct walk; float32: the counting walk is direct,
-// with the same bits).
-bool walk_lists(const hts_ctx *c)
+// Whether launch_walk lists the interactions first, given the buffers (float64: a
+// depth that was asked for is the cut of the direct walk; float32: the counting
+// walk is direct, with the same bits).
+bool walk_wants_lists(const hts_ctx *c)
 {
     const bool fp64 = c->cfg.precision == HTS_FP64;
     return c->nseg == 1 && (fp64 ? c->walk_split < 0 : !c->counters_on) && list_units(c->n, fp64) > 0;
 }
+
+bool walk_lists(const hts_ctx *c) { return c->list_entries && walk_wants_lists(c); }
 
 void launch_walk(hts_ctx *c)
 {
