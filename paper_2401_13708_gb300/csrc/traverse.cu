@@ -1467,10 +1467,12 @@ struct ExactArgs {
     const int64_t *seg_off;
 };
 
-__device__ __forceinline__ void exact_ranges(const ExactArgs &A, int i, int &jlo, int &jhi, int &cbeg, int &cend)
+// Own segment [jlo, jhi); the union over the block's threads, cut into chunks
+// [cbeg, cend).  Returns whether the block's points share one segment.
+__device__ __forceinline__ bool exact_ranges(const ExactArgs &A, int i, int &jlo, int &jhi, int &cbeg, int &cend)
 {
-    // own segment [jlo, jhi); the union over the block's threads, cut into chunks
     int blo = 0, bhi = A.n;
+    bool one = true;
     jlo = 0;
     jhi = A.n;
     if (A.seg_of) {
@@ -1480,24 +1482,25 @@ __device__ __forceinline__ void exact_ranges(const ExactArgs &A, int i, int &jlo
         jhi = (int)A.seg_off[si + 1];
         blo = (int)A.seg_off[A.seg_of[first]];
         bhi = (int)A.seg_off[A.seg_of[last] + 1];
+        one = A.seg_of[first] == A.seg_of[last];
     }
     const int tiles = (bhi - blo + kExactBlock - 1) / kExactBlock;
     const int per = (tiles + A.split - 1) / A.split;
     cbeg = min(bhi, blo + (int)blockIdx.y * per * kExactBlock);
     cend = min(bhi, cbeg + per * kExactBlock);
+    return one;
 }
 
-// Adds one exact pair (weight 0 unless `take`).
+// Adds one exact pair.
 template <int GF>
-__device__ __forceinline__ void add_exact_f32(float2 qh, float2 ql, float twoil, const PointF &o, bool take, float2 &rxy,
-                                              float2 &rsz)
+__device__ __forceinline__ void add_exact_f32(float2 qh, float2 ql, float twoil, const PointF &o, float2 &rxy, float2 &rsz)
 {
     const float2 d = delta2(qh, ql, make_float2(o.xh, o.yh), make_float2(o.xl, o.yl));
     const float s = fmaf(d.x, d.x, d.y * d.y);
     const PairF t = pair_terms_f32<GF>(s * twoil * o.il);
-    const float kk = take ? t.rep * o.il : 0.0f;
+    const float kk = t.rep * o.il;
     rxy = __ffma2_rn(make_float2(kk, kk), d, rxy);
-    rsz = __ffma2_rn(make_float2(kk, take ? 1.0f : 0.0f), make_float2(s, t.w), rsz);
+    rsz = __ffma2_rn(make_float2(kk, 1.0f), make_float2(s, t.w), rsz);
 }
 
 template <int GF>
@@ -1507,7 +1510,7 @@ __global__ void __launch_bounds__(kExactBlock) exact_f32_kernel(const PointF *__
     const int n = A.n;
     const int i = blockIdx.x * kExactBlock + threadIdx.x;
     int jlo, jhi, cbeg, cend;
-    exact_ranges(A, i, jlo, jhi, cbeg, cend);
+    const bool one = exact_ranges(A, i, jlo, jhi, cbeg, cend);
     const PointF q = pts[i < n ? i : n - 1];
     const float2 qh = make_float2(q.xh, q.yh), ql = make_float2(q.xl, q.yl);
     const float twoil = 2.0f * q.il;
@@ -1517,18 +1520,27 @@ __global__ void __launch_bounds__(kExactBlock) exact_f32_kernel(const PointF *__
         if (j < cend) tile[threadIdx.x] = pts[j];
         __syncthreads();
         const int cnt = min(kExactBlock, cend - base);
-        // every pair of a full tile off the diagonal and inside the segment
-        // counts: no tests, four pairs in flight (a pair that does not count
-        // is added with weight 0 otherwise)
-        const bool plain = cnt == kExactBlock && !A.seg_of && (base + cnt <= blockIdx.x * kExactBlock ||
+        // every pair of a full tile off the diagonal counts where the block's
+        // points share one segment: no tests.  Otherwise the sums keep their
+        // values where a pair does not count (with weight 0 a point that is not
+        // finite would reach other segments: 0 x NaN is NaN).  Four pairs in
+        // flight either way: a block on a boundary passes over both segments and
+        // decides the kernel's time (two segments of 30,000 points: 4.9 ms with a
+        // branch around the pair)
+        const bool plain = cnt == kExactBlock && one && (base + cnt <= blockIdx.x * kExactBlock ||
                                                                base >= (blockIdx.x + 1) * kExactBlock);
         if (plain) {
 #pragma unroll 4
-            for (int k = 0; k < kExactBlock; ++k) add_exact_f32<GF>(qh, ql, twoil, tile[k], true, rxy, rsz);
+            for (int k = 0; k < kExactBlock; ++k) add_exact_f32<GF>(qh, ql, twoil, tile[k], rxy, rsz);
         } else {
+#pragma unroll 4
             for (int k = 0; k < cnt; ++k) {
                 const int jj = base + k;
-                add_exact_f32<GF>(qh, ql, twoil, tile[k], jj != i && jj >= jlo && jj < jhi, rxy, rsz);
+                const bool take = jj != i && jj >= jlo && jj < jhi;
+                float2 u = rxy, v = rsz;
+                add_exact_f32<GF>(qh, ql, twoil, tile[k], u, v);
+                rxy = make_float2(take ? u.x : rxy.x, take ? u.y : rxy.y);
+                rsz = make_float2(take ? v.x : rsz.x, take ? v.y : rsz.y);
             }
         }
         __syncthreads();
