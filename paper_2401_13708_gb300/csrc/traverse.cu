@@ -653,7 +653,7 @@ __device__ __forceinline__ void sum_batch_f32(LaneF &L, const BatchF &B, int bat
         T.yh[lane] = c.yh;
         T.xl[lane] = c.xl;
         T.yl[lane] = c.yl;
-        T.il[lane] = c.il;
+        T.il[lane] = have ? c.il : 0.0f;  // (past the count: weight 0 times a term that must be finite)
         T.count[lane] = c.count;
         unsigned bits = transpose_bits(mask, lane);
         __syncwarp();
