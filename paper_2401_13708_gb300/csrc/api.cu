@@ -103,14 +103,15 @@ void drop_lists(hts_ctx *c)
 }
 
 // Float32 node slots: one never written by a tree build reads as an empty bucket
-// (count 0), which the walk steps over (its skip is its index + 1).
+// (count 0), which the walk steps over (its skip is its index + 1).  In stream
+// order: a wait for the whole device fails while another thread captures a graph.
 int alloc_nodes32(hts_ctx *c, size_t N)
 {
     const int64_t slots = (int64_t)(2 * N + kWalkOverrun);
     int r = dalloc(c, &c->nodes32, (size_t)slots);
     if (r) return r;
-    empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256>>>(slots, c->nodes32);
-    if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return HTS_ECUDA;
+    empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256, 0, c->stream>>>(slots, c->nodes32);
+    LAUNCHED("empty_nodes");
     return HTS_OK;
 }
 
