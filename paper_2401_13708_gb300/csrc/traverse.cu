@@ -356,6 +356,11 @@ __device__ __forceinline__ bool visit_ancestors_f32(const Cut &F, bool live, int
     return live;
 }
 
+// 0, or NaN for a point that is not finite.  No criterion and so no other point
+// takes such a point's leaf; through its Z_i the embedding's Z is NaN, and with
+// it the gradient of every point (as the exact one).
+__device__ __forceinline__ double zero_if_finite(double x, double y) { return (x - x) + (y - y); }
+
 // A chunk's sums into its points' results (or, split, into the partial sums
 // of subtree `sum`).
 __device__ __forceinline__ void store_lane(const LaneF &L, int sum, int n, const uint32_t *__restrict__ idx,
@@ -371,7 +376,7 @@ __device__ __forceinline__ void store_lane(const LaneF &L, int sum, int n, const
     double il = 0.5 * (double)L.twoil;
     double rsd = il * (double)L.rsz.x;
     frep[i] = make_double2(4.0 * il * ((double)L.rxy.x + rsd * x), 4.0 * il * ((double)L.rxy.y + rsd * y));
-    zi[i] = (double)L.rsz.y;
+    zi[i] = (double)L.rsz.y + zero_if_finite(x, y);
 }
 
 // One visit of the direct walk's cursor at `node`, whose data `c` are loaded:
@@ -970,7 +975,7 @@ __device__ __forceinline__ void store_lane(const LaneD &L, int sum, int n, const
     const uint32_t i = idx[L.p];
     const double il = 0.5 * L.twoil, rsd = il * L.rs;
     frep[i] = make_double2(4.0 * il * (L.rx + rsd * L.x), 4.0 * il * (L.ry + rsd * L.y));
-    zi[i] = L.z;
+    zi[i] = L.z + zero_if_finite(L.x, L.y);
 }
 
 // One warp walks for a chunk (sum `sum` of the cut when there are partial sums).
@@ -1449,7 +1454,7 @@ __global__ void __launch_bounds__(kCombineBlock) walk_combine_kernel(int n, cons
     const double rsd = il * rs;
     const uint32_t i = idx ? idx[p] : (uint32_t)p;  // sorted positions, or points
     frep[i] = make_double2(4.0 * il * (rx + rsd * x), 4.0 * il * (ry + rsd * y));
-    zi[i] = z;
+    zi[i] = z + zero_if_finite(x, y);
 }
 
 // Exact repulsion: one thread per point i, tiles of kExactBlock points j

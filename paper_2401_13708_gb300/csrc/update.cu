@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     if (!A.seg_of) {  // one problem: 1 / Z once per block (float64 division is costly here)
         if (threadIdx.x == 0) {
             const double Z0 = A.Z[0];
-            s_invz = Z0 > 0.0 ? 4.0 * (1.0 / Z0) : 0.0;
+            s_invz = Z0 <= 0.0 ? 0.0 : 4.0 * (1.0 / Z0);  // (NaN stays NaN: a point is not finite)
         }
         __syncthreads();
     }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kBlock) update_kernel(UpdateArgs A)
     double invZ4;  // 4 / Z
     if (A.seg_of) {
         const double Z = A.Z[sg];
-        invZ4 = Z > 0.0 ? 4.0 * (1.0 / Z) : 0.0;
+        invZ4 = Z <= 0.0 ? 0.0 : 4.0 * (1.0 / Z);
     } else {
         invZ4 = s_invz;
     }

@@ -41,3 +41,22 @@ def test_exact_gradient_of_the_other_embedding(precision):
     # the same terms in float32 (float64) sums of another order: 110 roundings each
     eps = 2.0 ** (-24 if precision == "fp32" else -53)
     assert np.linalg.norm(g[90:] - h) <= 110.0 * 8.0 * eps * np.linalg.norm(h)
+
+
+# listed, direct (float32 above 32,768 points; a depth in float64), and the
+# embedding beside it in a batch
+@pytest.mark.parametrize("precision,n,depth", [("fp32", 2000, -1), ("fp32", 33000, -1), ("fp64", 2000, -1),
+                                               ("fp64", 2000, 0), ("fp64", 12000, -1)])
+def test_tree_gradient_of_its_own_embedding(precision, n, depth):
+    t, y = diverged(precision, n, 17, 0.0)
+    with t:
+        t.set_walk_split(depth)
+        g, z = t.grad(0.5)
+        assert not np.isfinite(g).any() and not np.isfinite(z)
+    off = np.array([0, 90, n])
+    t, y = diverged(precision, n, 80, 0.0, off)
+    with t:
+        g, _ = t.grad(0.5)
+        z = t.segment_Z()
+    assert np.isfinite(g[90:]).all() and np.isfinite(z[1])
+    assert not np.isfinite(g[:90]).any() and not np.isfinite(z[0])
