@@ -63,6 +63,18 @@ __host__ __device__ __forceinline__ float rcp_near(float x)  // 1 / x within 2^-
 #endif
 }
 
+// a b rounded, whatever is done with it: a product whose rounding error is taken
+// off elsewhere must not be fused into a sum
+__host__ __device__ __forceinline__ float product(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    volatile float p = a * b;
+    return p;
+#endif
+}
+
 __host__ __device__ __forceinline__ Pair32 pair_of(double x)
 {
     Pair32 p;
@@ -97,11 +109,11 @@ __host__ __device__ __forceinline__ bool quantise_angle(double x, double y, int 
     const int k = (int)(t0 * 64.0f + 0.5f);  // 0 .. 64
     const float c = (float)k * (1.0f / 64.0f);
     // numerator min - c max (the first difference is exact: c max is within half of min, or 0)
-    const float p = c * mx.h, pe = fmaf(c, mx.h, -p);
+    const float p = product(c, mx.h), pe = fmaf(c, mx.h, -p);
     const float a = mn.h - p, b = mn.l - pe - c * mx.l;
     const float nh = a + b, nl = b - (nh - a);
     // denominator max + c min
-    const float p2 = c * mn.h, p2e = fmaf(c, mn.h, -p2);
+    const float p2 = product(c, mn.h), p2e = fmaf(c, mn.h, -p2);
     const float dh = mx.h + p2, dl = ((mx.h - dh) + p2) + p2e + mx.l + c * mn.l;
     const float rc = rcp_near(dh);
     const float q0 = nh * rc;
