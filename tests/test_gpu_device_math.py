@@ -1,11 +1,14 @@
-"""csrc/polar.cuh as the device runs it (the host build of the other tests has other
-roundings to choose from): wherever the float pairs decide a coordinate they
-give the float64 definition's value, and they decide nearly always."""
+"""csrc/polar.cuh and csrc/f64math.cuh as the device runs them (the host builds of
+the other tests have other roundings to choose from, and other seeds): wherever
+the float pairs decide a coordinate they give the float64 definition's value,
+and they decide nearly always; the float64 functions keep the bounds of
+test_f64math_host.py."""
 import math
 import os
 import shutil
 import struct
 import subprocess
+from decimal import Decimal, getcontext
 
 import numpy as np
 import pytest
@@ -41,6 +44,11 @@ def keys_build(tmp_path_factory):
     return compiled(tmp_path_factory.mktemp("keys"))
 
 
+@pytest.fixture(scope="module")
+def walk_build(tmp_path_factory):
+    return compiled(tmp_path_factory.mktemp("walk"), "-ftz=true")  # (as traverse.cu)
+
+
 def quantise(u):
     return min(max(math.floor(u * 2.0 ** 29), 0), 2 ** 29 - 1)
 
@@ -71,3 +79,24 @@ def test_decided_coordinates_are_the_definition(keys_build, r0, r1, area):
             sure_r += 1
     assert sure_a > n - 1000  # (all but those put on steps and lines)
     assert sure_r > n - 100 if hi - lo >= hi / 4.0 else sure_r == 0
+
+
+def test_float64_functions_in_units_of_the_last_place(walk_build):
+    getcontext().prec = 40
+    rng = np.random.default_rng(4)
+    xs = list(10.0 ** rng.uniform(-36, 33, 1500)) + list(10.0 ** rng.uniform(-3, 1, 1500))
+    edges = [(1.0 + (j + 0.5) / 128.0) * 2.0 ** k for j in range(128) for k in (0, 1, 30)]
+    xs += [e - 1.0 for e in edges] + [np.nextafter(e, 0.0) for e in edges] + [1.0 + 2.0 ** -k for k in range(1, 50)]
+    xs += [4e-300, 2.0 ** -127, 2.0 ** 126, np.nextafter(2.0 ** -127, 0.0), np.nextafter(2.0 ** 127, 0.0)]
+    low = [5e-324, 1e-310, 2.0 ** 127, 2.0 ** 128, 1e300]  # (log alone: the library's outside its tables)
+    xs = [float(x) for x in xs + low if x > 0.0]
+    for k, (x, row) in enumerate(zip(xs, walk_build("math", ["%s\n" % bits(x) for x in xs]))):
+        t, rs, rc, l1, lx = (struct.unpack("<d", struct.pack("<Q", v))[0] for v in row)
+        d = Decimal(x)
+        want = {"log": (lx, d.ln(), 3)}
+        if k < len(xs) - len(low):
+            want.update({"sqrt": (t, d.sqrt(), 2), "rsqrt": (rs, 1 / d.sqrt(), 2), "reciprocal": (rc, 1 / d, 2),
+                         "log1p": (l1, (1 + d).ln() if x > 1e-12 else d - d * d / 2 + d * d * d / 3, 3)})
+        for name, (got, ref, limit) in want.items():
+            err = abs(Decimal(got) - ref) * 2 ** 53
+            assert err <= limit * abs(ref), (name, x, got)
