@@ -39,3 +39,16 @@ def test_listed_against_direct(n, rho, theta):
         g2, z2 = t.grad(theta)
     assert abs(z - z2) <= 1e-12 * abs(z2)
     assert np.linalg.norm(g - g2) <= 1e-12 * np.linalg.norm(g2) + 1e-300
+
+
+@pytest.mark.parametrize("n,listed", [(262144, True), (262145, False)])
+def test_limit_of_the_float64_lists(n, listed):
+    with HyperbolicTSNE(precision="fp64") as t:
+        t.set_P(np.zeros(n + 1, np.int64), np.zeros(0, np.int32), np.zeros(0, np.float64))
+        t.set_Y(inputs.spread_embedding(np.arange(n) % 37, 3, rho_hi=9.0))
+        g, z = t.grad(0.8)
+        t.set_walk_split(0)
+        g2, z2 = t.grad(0.8)
+    assert np.array_equal(g, g2) is not listed
+    assert abs(z - z2) <= n * 2.0 ** -53 * abs(z2)
+    assert np.linalg.norm(g - g2) <= n * 2.0 ** -53 * np.linalg.norm(g2)
