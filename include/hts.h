@@ -195,8 +195,8 @@ HTS_API int hts_get_tree(hts_ctx *ctx, int64_t cap, int64_t *count_out, int32_t 
 
 /* Counters (host int64[5]): [0..3] summed over the tree walks run while
  * counting is on -- accepted cells, leaf pair interactions, warp node
- * visits, query points (the walk then runs a counting variant; switching
- * counting on resets them); [4] the number of CUDA kernels this context
+ * visits, query points (the walk then runs a counting variant, with the same
+ * results; switching counting on resets them); [4] the number of CUDA kernels this context
  * has launched. */
 HTS_API int hts_get_counters(hts_ctx *ctx, int64_t *out5);
 HTS_API int hts_set_counters(hts_ctx *ctx, int enable);

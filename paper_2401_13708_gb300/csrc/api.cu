@@ -3,7 +3,8 @@
 // One iteration (hts_step) queues, on the context's stream:
 //   prep_points -> make_keys -> sort -> build_tree -> walk -> reduce_z -> update
 // with attract beside the tree build and the walk, or, for theta == 0, prep_points -> exact -> attract -> reduce_z -> update.
-// Nothing is allocated and nothing is copied to the host inside the loop;
+// Nothing is allocated (but what only a walk needs, by the first one: ensure_lists,
+// ensure_nodes) and nothing is copied to the host inside the loop;
 // the status word is read once after the last iteration.
 #include <math.h>
 #include <stdio.h>
@@ -198,9 +199,10 @@ int ensure_points(hts_ctx *c, int64_t n)
 // nodes, which decide its criterion (64 bytes a point), and the interaction
 // lists (up to 175 MB at 32,768 points in float32, 570 MB at 262,144 in
 // float64).  run_gradient asks for the lists once the tree build is queued, so
-// that their allocation runs beside it (N = 20,011: the first gradient takes 48 us
-// more, hts_set_Y before it 50 us less than with the lists taken there).  Lists that do not fit
-// are left out until the size changes: the walk is then the direct one.
+// that their allocation runs beside it (N = 20,011: the first gradient takes
+// 48 us more, hts_set_Y before it 50 us less than with the lists taken there).
+// Lists that do not fit are left out until the size changes: the walk is then
+// the direct one.
 int ensure_nodes(hts_ctx *c)
 {
     if (c->nodes32 || c->n == 0) return HTS_OK;
