@@ -3,8 +3,8 @@
 // One iteration (hts_step) queues, on the context's stream:
 //   prep_points -> make_keys -> sort -> build_tree -> walk -> reduce_z -> update
 // with attract beside the tree build and the walk, or, for theta == 0, prep_points -> exact -> attract -> reduce_z -> update.
-// Nothing is allocated (but what only a walk needs, by the first one: ensure_lists,
-// ensure_nodes) and nothing is copied to the host inside the loop;
+// Nothing is allocated (but the interaction lists, by the first walk that wants
+// them: ensure_lists) and nothing is copied to the host inside the loop;
 // the status word is read once after the last iteration.
 #include <math.h>
 #include <stdio.h>
@@ -103,19 +103,6 @@ void drop_lists(hts_ctx *c)
     c->lists_refused = 0;
 }
 
-// Float32 node slots: one never written by a tree build reads as an empty bucket
-// (count 0), which the walk steps over (its skip is its index + 1).  In stream
-// order: a wait for the whole device fails while another thread captures a graph.
-int alloc_nodes32(hts_ctx *c, size_t N)
-{
-    const int64_t slots = (int64_t)(2 * N + kWalkOverrun);
-    int r = dalloc(c, &c->nodes32, (size_t)slots);
-    if (r) return r;
-    empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256, 0, c->stream>>>(slots, c->nodes32);
-    LAUNCHED("empty_nodes");
-    return HTS_OK;
-}
-
 int ensure_points(hts_ctx *c, int64_t n)
 {
     if (n == c->cap_n && (c->pts32 || c->pts64)) return HTS_OK;
@@ -135,14 +122,20 @@ int ensure_points(hts_ctx *c, int64_t n)
         AL(c->pts32, N);
         AL(c->apts32, N);
         AL(c->spts32, N);
-        if ((r = alloc_nodes32(c, N))) return r;
     } else {
         AL(c->pts64, N);
         AL(c->spts64, N);
         AL(c->nodes64, 2 * N);
-        dfree(&c->nodes32);
     }
-    drop_lists(c);  // (and float64 mode's float32 nodes: ensure_nodes)
+    // float32 nodes (in float64 mode they decide the criterion): a slot never
+    // written by a tree build reads as an empty bucket (count 0), which the walk
+    // steps over (its skip is its index + 1).  In stream order: a wait for the
+    // whole device fails while another thread captures a graph.
+    const int64_t slots = (int64_t)(2 * N + kWalkOverrun);
+    AL(c->nodes32, (size_t)slots);
+    empty_nodes_kernel<<<(unsigned)((slots + 255) / 256), 256, 0, c->stream>>>(slots, c->nodes32);
+    LAUNCHED("empty_nodes");
+    drop_lists(c);  // (taken again by the first walk that wants them: ensure_lists)
     if (c->nodes64 && cudaMemset(c->nodes64, 0, sizeof(NodeD) * 2 * N) != cudaSuccess) return HTS_ECUDA;
     AL(c->keys, N);
     AL(c->keys_alt, N);
@@ -194,22 +187,13 @@ int ensure_points(hts_ctx *c, int64_t n)
     return HTS_OK;
 }
 
-// What a tree walk needs beyond ensure_points' buffers is taken by the first call
-// that walks (theta = 0 never does, segments never list): float64 mode's float32
-// nodes, which decide its criterion (64 bytes a point), and the interaction
-// lists (up to 175 MB at 32,768 points in float32, 570 MB at 262,144 in
-// float64).  run_gradient asks for the lists once the tree build is queued, so
-// that their allocation runs beside it (N = 20,011: the first gradient takes
+// The interaction lists (up to 175 MB at 32,768 points in float32, 570 MB at
+// 262,144 in float64) are taken by the first walk that lists: exact gradients and
+// segments never do.  run_gradient asks for them once the tree build is queued,
+// so that their allocation runs beside it (N = 20,011: the first gradient takes
 // 48 us more, hts_set_Y before it 50 us less than with the lists taken there).
 // Lists that do not fit are left out until the size changes: the walk is then
 // the direct one.
-int ensure_nodes(hts_ctx *c)
-{
-    if (c->nodes32 || c->n == 0) return HTS_OK;
-    c->layout_version += 1;
-    return alloc_nodes32(c, (size_t)c->n);
-}
-
 void ensure_lists(hts_ctx *c)
 {
     if (c->list_entries || c->lists_refused || !walk_wants_lists(c)) return;
@@ -301,7 +285,6 @@ int run_gradient(hts_ctx *c, double theta, cudaEvent_t *ev = nullptr)
         launch_exact(c);
         LAUNCHED("exact");
     } else {
-        if ((r = ensure_nodes(c))) return r;
         if (attract && fork_at == 0 && (r = fork_attract())) return r;
         launch_make_keys(c);
         LAUNCHED("make_keys");
@@ -385,11 +368,7 @@ void drop_graph(hts_ctx *c)
 // stream, unless the cached graph already matches the arguments and layout.
 int capture_iteration(hts_ctx *c, double theta, double exag, double lr, double mom)
 {
-    if (theta > 0.0) {  // (nothing is allocated in a capture)
-        const int r = ensure_nodes(c);
-        if (r) return r;
-        ensure_lists(c);
-    }
+    if (theta > 0.0) ensure_lists(c);  // (nothing is allocated in a capture)
     const double key[5] = {theta, exag, lr, mom, (double)c->layout_version};
     if (c->gexec && memcmp(key, c->gkey, sizeof(key)) == 0) return HTS_OK;
     drop_graph(c);
@@ -1239,7 +1218,6 @@ int hts_autotune(hts_ctx *c, double theta, int reps, int *tuning)
         c->walk_split = -1;  // (with the lists: the depths are timed below)
         if (theta > 0.0) ensure_lists(c);
         c->walk_split = keep_split;
-        if (theta > 0.0 && (r = ensure_nodes(c))) return r;
         cudaEvent_t a = c->events[0], b = c->events[1];
         launch_prep_points(c);
         LAUNCHED("prep_points");

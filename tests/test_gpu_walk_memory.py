@@ -1,6 +1,6 @@
-"""The interaction lists, and float64 mode's float32 nodes, are taken by the first
-call that walks a tree with them: not by a context that only computes exact
-gradients, and not by batches, which never list."""
+"""The interaction lists are taken by the first call that walks a tree with them:
+not by a context that only computes exact gradients, and not by batches, which
+never list."""
 import numpy as np
 import pytest
 
@@ -24,10 +24,9 @@ def context(n, precision):
     return t
 
 
-# lists: 175 MB at 32,768 points in float32; 268 MB (and 4 MB of nodes) at
-# 32,768 in float64, by the sizes of list_pages
-@pytest.mark.parametrize("precision,least", [("fp32", 160 * MB), ("fp64", 160 * MB)])
-def test_lists_are_taken_by_the_first_listed_walk(precision, least):
+# lists: 175 MB at 32,768 points, by the sizes of list_pages
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_lists_are_taken_by_the_first_listed_walk(precision):
     n = 32768
     with context(n, precision) as t:  # (kernels are loaded, pools warm)
         for theta in (0.0, 0.5):
@@ -41,7 +40,7 @@ def test_lists_are_taken_by_the_first_listed_walk(precision, least):
         g2, z2 = t.grad(0.5)
         assert free() == f2
         assert np.array_equal(g, g2) and z == z2
-    assert f0 - f1 < 8 * MB and f1 - f2 > least
+    assert f0 - f1 < 8 * MB and f1 - f2 > 160 * MB
 
 
 def test_batches_take_no_lists():
